@@ -533,6 +533,8 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
     p->wdt = w_dtype;
     p->xdt = x_dtype;
     p->kernel = kernel;
+    // an explicit PLAIN stays the plain kernel
+    p->f32_blocks = kernel == SPMM_KERNEL_PLAIN && o.kernel == SPMM_KERNEL_AUTO;
     p->host_only = o.host_only != 0;
     p->sm_count = 152;
     if (!p->host_only) {
@@ -809,7 +811,10 @@ static spmm_status launch_product(spmm_plan *p, const void *d_X, int64_t n, int6
                                   void *d_Y, int64_t ldy, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     switch (p->kernel) {
-        case SPMM_KERNEL_PLAIN: e = launch_plain(p, d_X, n, ldx, d_Y, ldy, s); break;
+        case SPMM_KERNEL_PLAIN:
+            e = p->f32_blocks ? launch_f32(p, d_X, n, ldx, d_Y, ldy, s)
+                              : launch_plain(p, d_X, n, ldx, d_Y, ldy, s);
+            break;
         case SPMM_KERNEL_GATHER: e = launch_gather(p, d_X, n, ldx, d_Y, ldy, s); break;
         case SPMM_KERNEL_TC: e = launch_tc(p, d_X, n, ldx, d_Y, ldy, s); break;
         case SPMM_KERNEL_BGATHER: e = launch_bgather(p, d_X, n, ldx, d_Y, ldy, s); break;

@@ -722,9 +722,10 @@ cudaError_t launch_pack_csr(const spmm_plan *p, const void *d_values, const int3
     const unsigned g = grid1d(total, 256) > 4096u ? 4096u : grid1d(total, 256);
     const int32_t *st = d_nnzb ? p->d_status : nullptr;
     switch (dtype_size(p->wdt)) {
-        case 4:
+        case 4:   // (the FP32 block kernel reads its blocks column by column)
             pdl_launch(pack_csr_kernel<uint32_t>, dim3(g), dim3(256), 0, s,
-                (const uint32_t *)d_values, p->d_perm, nmax, p->b, p->transposed ? 1 : 0, d_nnzb, st,
+                (const uint32_t *)d_values, p->d_perm, nmax, p->b,
+                p->transposed != p->f32_blocks ? 1 : 0, d_nnzb, st,
                 (uint32_t *)p->d_packed);
             break;
         case 2:

@@ -129,6 +129,8 @@ struct spmm_plan {
     int tc_geo = 0;                // TC stage geometry: 0 dense tiles, 1 sparse tiles
     int col_tiles = 0;             // TC: column tiles per CTA, 0 automatic (launch-time choice)
     int64_t groups = 0;            // static TC: near-equal tile-row groups (0: equal partition by R)
+    bool f32_blocks = false;       // FP32 b >= 4 plans AUTO chose: the block kernel (k_f32.cu),
+                                   // values packed column by column within each block
     bool transposed = false;       // applies W^T: values arrive as W's blocks, packed transposed
     int32_t *d_sd_items = nullptr; // b = 16: SDDMM work items (count, then (row, e0, e1) triples)
     int64_t sd_items_cap = 0;
@@ -180,6 +182,9 @@ cudaError_t launch_pack_tiles(const spmm_plan *p, const void *d_values, const fl
                               const int32_t *d_nnzb, cudaStream_t s);
 cudaError_t launch_plain(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
                          int64_t ldy, cudaStream_t s);
+// FP32 blocks, b >= 4 (k_f32.cu); launch_plain is the one-thread-per-output kernel
+cudaError_t launch_f32(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
+                       int64_t ldy, cudaStream_t s);
 cudaError_t launch_gather(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
                           int64_t ldy, cudaStream_t s);
 // dense rows (ld = n) of 2- or 4-byte values -> stride ld, on the device
