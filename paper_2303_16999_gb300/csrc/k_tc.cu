@@ -267,9 +267,13 @@ struct TcProb {
 };
 
 // A stage whose entries are 2 to 4 consecutive tile columns (record info
-// bit 20) gets its X slabs in one TMA box of 4 slabs when X's map is 3-D;
-// the slabs then lie 2048 B apart inside each 64-column half, the halves
-// 8192 B apart.
+// bit 20) gets its X slabs in one TMA box of 4 slabs, or with a 2-D map (n not
+// a multiple of 64) in one box per 64-column half; the slabs then lie 2048 B
+// apart inside each half, the halves 8192 B apart.  A box costs about 110
+// cycles of an SM's TMA unit whatever its size, so eight 2 KB boxes per stage
+// bound the dense-tile plans with a 2-D map: 4096 x 4096, b = 4, d = 1/8, in
+// 16-row groups split along k, n = 24: 20.4 -> 14.7 us, n = 100: 19.8 -> 17.0;
+// 4096 x 16384, b = 8, d = 1/8, n = 200: 45.2 -> 39.7.
 
 struct TcBatch {
     CUtensorMap maps[kMaxBatch]; // X of each problem
@@ -432,6 +436,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                 const int h = (nent + 1) >> 1;
                 const int xlo = pid == 2 ? h : 0, mine = pid == 2 ? nent - h : h;
                 const uint32_t col = __shfl_sync(0xffffffffu, rc, min(3 + xlo + lane, kRecWords - 1));
+                const uint32_t jcol = __shfl_sync(0xffffffffu, rc, 3);   // the stage's first column
                 int w = 1;
                 if (lane == 0) w = mbar_wait(&sm->empty[stage], phase ^ 1, sm, B.wait_ns) ? 1 : 0;
                 if (!__shfl_sync(0xffffffffu, w, 0)) return -1;
@@ -467,7 +472,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                     // first warp of the tile) or one box per slab, with a 2-D
                     // map as two 64-column boxes per slab (the lower one only
                     // when the upper 64 columns lie past n)
-                    const bool joint = (info & kJointBit) && P.x3d;
+                    const bool joint = (info & kJointBit) != 0;
                     const int tset = (pid - 1) & 1, part = (pid - 1) >> 1;
                     const bool act = tset == 0 || two;
                     const int per = (nent + G::xprod - 1) / G::xprod;
@@ -490,6 +495,12 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                         if (act && !joint && lane < cnt)
                             tma_load_3d(xs + (lo + lane) * kSlabBytes, &B.maps[un.p], 0,
                                         (int)xc * kTile, nh, &sm->full[stage]);
+                    } else if (joint) {
+                        // 2-D map: one box of slabs per 64-column half
+                        if (act && cnt && lane < (half ? 1 : 2))
+                            tma_load_2d(xs + lane * kJointSlabs * (kSlabBytes / 2), &B.maps4[un.p],
+                                        (int)ncol + lane * (kNTile / 2),
+                                        (int)jcol * kTile, &sm->full[stage]);
                     } else if (act && lane < cnt) {
                         uint8_t *slab = xs + (lo + lane) * kSlabBytes;
                         tma_load_2d(slab, &B.maps[un.p], (int)ncol, (int)xc * kTile, &sm->full[stage]);
@@ -497,13 +508,21 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                             tma_load_2d(slab + kSlabBytes / 2, &B.maps[un.p], (int)ncol + kNTile / 2,
                                         (int)xc * kTile, &sm->full[stage]);
                     }
-                } else if ((info & kJointBit) && P.x3d) {
-                    // consecutive columns: X producer 1 requests all slabs in one box
+                } else if (info & kJointBit) {
+                    // consecutive columns: X producer 1 requests all slabs in one
+                    // box, or with a 2-D map each producer those of one 64-column
+                    // half (the upper one only if it holds columns of n)
+                    const int x0 = n0 + (pid == 2 ? kNTile / 2 : 0);
                     if (lane == 0) {
-                        if (pid == 1) {
-                            mbar_arrive_tx(&sm->full[stage], kJointSlabs * kSlabBytes);
-                            tma_load_3d(st, &B.maps4[un.p], 0, (int)col * kTile, n0 / (kNTile / 2),
-                                        &sm->full[stage]);
+                        if (P.x3d ? pid == 1 : x0 < P.n) {
+                            mbar_arrive_tx(&sm->full[stage],
+                                           kJointSlabs * (P.x3d ? kSlabBytes : kSlabBytes / 2));
+                            if (P.x3d)
+                                tma_load_3d(st, &B.maps4[un.p], 0, (int)jcol * kTile,
+                                            n0 / (kNTile / 2), &sm->full[stage]);
+                            else
+                                tma_load_2d(st + (pid == 2 ? kJointSlabs * (kSlabBytes / 2) : 0),
+                                            &B.maps4[un.p], x0, (int)jcol * kTile, &sm->full[stage]);
                         } else {
                             mbar_arrive(&sm->full[stage]);
                         }
@@ -614,7 +633,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                 last = (info >> 31) != 0;
                 const uint32_t myword = sm->meta[stage].prog[half][lane];   // words >= nmma unused
                 const uint32_t sbase = smem_u32(stages + stage * G::bytes);
-                const bool joint = (info & kJointBit) && B.prob[un.p].x3d;
+                const bool joint = (info & kJointBit) != 0;
                 const uint64_t adesc0 = joint ? a_desc_joint(sbase) : a_desc(sbase);
                 const uint32_t astep = joint ? (kSlabBytes / 2) >> 4 : kSlabBytes >> 4;
                 const uint64_t bdesc0 = b_desc(sbase + G::w16);

@@ -20,9 +20,9 @@ constexpr int kRecWords = 16;           // words per stage record
 constexpr int kMmaStage = 32;           // MMAs per stage and row half (one per lane)
 constexpr int kJointSlabs = 4;          // slabs of a joint X box
 // A stage whose entries are 2 to 4 consecutive tile columns (record info
-// bit 20) gets its X slabs in one TMA box of kJointSlabs slabs when X's map
-// is 3-D; the slabs then lie 2048 B apart inside each 64-column half, the
-// halves 8192 B apart.
+// bit 20) gets its X slabs in one TMA box of kJointSlabs slabs (with a 2-D X
+// map one box per 64-column half); the slabs then lie 2048 B apart inside each
+// 64-column half, the halves 8192 B apart.
 constexpr uint32_t kJointBit = 1u << 20;
 constexpr int kBuildWarps = 16;         // warps of a stage_build_kernel CTA
 

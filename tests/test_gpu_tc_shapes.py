@@ -1,0 +1,49 @@
+"""Launch shapes of the static tensor-core plans, on integer-valued operands:
+sums of products are exact in FP32, so Y must equal the 64-bit product rounded
+once to the output type, whatever the groups, splits and column tiles.
+"""
+import numpy as np
+import pytest
+
+from paper_2303_16999_gb300 import spmm as S
+from paper_2303_16999_gb300 import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _problem(seed, m, k, n, b, nnzb, dt):
+    c = wl.integer_problem(seed, m, k, n, b, nnzb)
+    vals = torch.from_numpy(c["vals"]).to(dt).cuda()
+    x = torch.full((k, (n + 7) // 8 * 8), float("nan"), dtype=dt, device="cuda")
+    x[:, :n] = torch.from_numpy(c["X"]).to(dt)
+    w = torch.zeros((m // b, k // b, b, b), dtype=torch.float64, device="cuda")
+    w[torch.from_numpy(c["brow"]).long(), torch.from_numpy(c["bcol"]).long()] = vals.double()
+    want = w.transpose(1, 2).reshape(m, k) @ x[:, :n].double()
+    return c, vals, x[:, :n], want.to(dt)
+
+
+def _run(c, vals, x, want, pad=0, **kw):
+    m, n = want.shape
+    p = S.Plan(c["m"], c["k"], n, c["b"], w_dtype=S.dtype_code(vals.dtype), brow=c["brow"],
+               bcol=c["bcol"], kernel="tc", **kw)
+    p.pack(vals)
+    y = torch.full((m, n + pad), float("nan"), dtype=want.dtype, device="cuda")
+    p.run(x, y[:, :n])
+    torch.cuda.synchronize()
+    info = p.info()
+    assert p.status() == 0
+    p.close()
+    assert torch.equal(y[:, :n], want)
+    assert torch.isnan(y[:, n:]).all()
+    return info
+
+
+@pytest.mark.parametrize("n", [1, 8, 63, 65, 72, 100, 127, 129, 191, 200, 257, 450])
+@pytest.mark.parametrize("geo,ct", [(1, 1), (2, 1), (1, 2), (2, 2)])
+def test_joint_boxes_with_2d_maps(n, geo, ct):
+    """Stages of consecutive tile columns (every tile present) with n not a
+    multiple of 64: one box of slabs per 64-column half, the upper half
+    absent where it lies past n; k ends inside a box (31 tile columns)."""
+    case = _problem(300 + n, 272, 496, n, 4, 68 * 124 // 2, torch.bfloat16)
+    _run(*case, rows_per_group=16, stage_geometry=geo, col_tiles=ct)
