@@ -821,7 +821,9 @@ static spmm_status launch_product(spmm_plan *p, const void *d_X, int64_t n, int6
         default: set_error("bad kernel"); return SPMM_ERR_ARG;
     }
     if (e == cudaSuccess && p->n_red > 0 && p->kernel != SPMM_KERNEL_PLAIN)
-        e = launch_reduce(p, n, d_Y, ldy, s);
+        e = p->kernel == SPMM_KERNEL_TC && p->mode == SPMM_STATIC
+                ? launch_reduce_tc(1, &p, &n, &d_Y, &ldy, s)
+                : launch_reduce(p, n, d_Y, ldy, s);
     if (e != cudaSuccess) return cuda_fail(e, "launch");
     return SPMM_OK;
 }
@@ -1149,13 +1151,10 @@ spmm_status spmm_batch_run(int32_t count, spmm_plan *const *plans, const void *c
     if (ng) e = launch_bgather_batch(ng, gp, gx, gn, glx, gy, gly, s);
     if (e == cudaSuccess && nt) e = launch_tc_batch(nt, tp, tx, tn, tlx, ty, tly, s, true);
     if (e != cudaSuccess) return cuda_fail(e, "batched launch");
+    if (nt) e = launch_reduce_tc(nt, tp, tn, ty, tly, s);
+    if (e != cudaSuccess) return cuda_fail(e, "batched reduction");
     for (int i = 0; i < count; ++i) {
-        spmm_plan *p = plans[i];
-        if (p->kernel == SPMM_KERNEL_TC && p->n_red > 0 && n[i] > 0) {
-            e = launch_reduce(p, n[i], d_Y[i], ldy ? ldy[i] : n[i], s);
-            if (e != cudaSuccess) return cuda_fail(e, "batched reduction");
-        }
-        spmm_status st = finish_call(p, s);
+        spmm_status st = finish_call(plans[i], s);
         if (st != SPMM_OK) return st;
     }
     return SPMM_OK;

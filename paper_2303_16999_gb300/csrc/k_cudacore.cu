@@ -601,6 +601,68 @@ __global__ void reduce_kernel(const int32_t *__restrict__ red, const int32_t *__
   }
 }
 
+// The same sums for static tensor-core plans, of every product of a call in
+// one launch.  A split group's partials are contiguous, rows x n per work
+// item, so a thread adds four consecutive values, one 16-byte load per
+// partial, all in flight together; the sums run in chunk order as above.
+// Block y is one split group of one product, block x a share of its values.
+// With one thread per value and one launch per product a split plan's call
+// paid 5.3 us for its reduction beyond the partials' bytes; this pays 2.1 (both
+// fitted over 1270 timed launches).
+struct RedProb {
+    const int32_t *red, *grp_row0, *grp_rows;
+    const float *ws;
+    const int64_t *ws_row0;
+    void *Y;
+    int64_t ldy;
+    int32_t n, base, yvec;       // base: first y of the product
+};
+struct RedBatch {
+    RedProb prob[kMaxBatchProblems];
+    int32_t nprob;
+};
+constexpr int kRedThreads = 256;
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads) reduce_tc_kernel(const __grid_constant__ RedBatch B) {
+    pdl_enter();
+    int p = 0;
+    while (p + 1 < B.nprob && B.prob[p + 1].base <= (int)blockIdx.y) ++p;
+    const RedProb &P = B.prob[p];
+    const int32_t *rd = P.red + ((int)blockIdx.y - P.base) * 3;
+    const int32_t g = rd[0], slot0 = rd[1], nch = rd[2];
+    const int64_t n = P.n, total = (int64_t)P.grp_rows[g] * kTile * n / 4;
+    T *Y = reinterpret_cast<T *>(P.Y) + (int64_t)P.grp_row0[g] * kTile * P.ldy;
+    // (the partials of a group's items follow one another)
+    const float4 *ws = reinterpret_cast<const float4 *>(P.ws + P.ws_row0[slot0] * n);
+    for (int64_t i = blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < total;
+         i += (int64_t)gridDim.x * kRedThreads) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c0 = 0; c0 < nch; c0 += 8) {
+            float4 v[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c0 + c < nch) v[c] = ws[(c0 + c) * total + i];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c0 + c < nch) a.x += v[c].x, a.y += v[c].y, a.z += v[c].z, a.w += v[c].w;
+        }
+        int64_t r = i * 4 / n, j = i * 4 - r * n;
+        const float o[4] = {a.x, a.y, a.z, a.w};
+        if (P.yvec) {
+            Pack<T, 4> q;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) q.v[e] = Vec<T>::from_f(o[e]);
+            *reinterpret_cast<Pack<T, 4> *>(Y + r * P.ldy + j) = q;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                Y[r * P.ldy + j] = Vec<T>::from_f(o[e]);
+                if (++j == n) j = 0, ++r;
+            }
+        }
+    }
+}
+
 inline unsigned grid1d(int64_t total, int threads) {
     int64_t g = (total + threads - 1) / threads;
     if (g < 1) g = 1;
@@ -759,6 +821,40 @@ cudaError_t launch_gather(const spmm_plan *p, const void *X, int64_t n, int64_t 
         case SPMM_BF16: return gather_dispatch<__nv_bfloat16>(p, X, n, ldx, Y, ldy, s);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_reduce_tc(int count, const spmm_plan *const *plans, const int64_t *n,
+                             void *const *Y, const int64_t *ldy, cudaStream_t s) {
+    RedBatch B;
+    B.nprob = 0;
+    int64_t reds = 0, most = 0;
+    const spmm_plan *any = nullptr;
+    for (int i = 0; i < count; ++i) {
+        const spmm_plan *p = plans[i];
+        if (p->n_red == 0 || n[i] == 0) continue;
+        const int64_t ly = ldy ? ldy[i] : n[i];
+        const int yvec = n[i] % 4 == 0 && ly % 4 == 0 && (uintptr_t)Y[i] % 8 == 0;
+        B.prob[B.nprob++] = RedProb{p->d_red, p->d_grp_row0, p->d_grp_rows, p->d_ws, p->d_ws_row0,
+                                    Y[i], ly, (int32_t)n[i], (int32_t)reds, yvec};
+        reds += p->n_red;
+        most = std::max(most, (int64_t)p->R * kTile * n[i] / 4);
+        any = p;
+    }
+    if (!any) return cudaSuccess;
+    if (reds > 65535) {   // the grid's y limit
+        for (int i = 0; i < count; ++i) {
+            const cudaError_t e = launch_reduce(plans[i], n[i], Y[i], ldy ? ldy[i] : n[i], s);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
+    const int64_t want = std::max<int64_t>(1, 16 * (int64_t)std::max(any->sm_count, 1) / reds);
+    const int64_t gx = std::max<int64_t>(
+        1, std::min<int64_t>(std::min<int64_t>((most + kRedThreads - 1) / kRedThreads, want), 1024));
+    const dim3 grid((unsigned)gx, (unsigned)reds);
+    if (any->xdt == SPMM_BF16)
+        return pdl_launch(reduce_tc_kernel<__nv_bfloat16>, grid, dim3(kRedThreads), 0, s, B);
+    return pdl_launch(reduce_tc_kernel<__half>, grid, dim3(kRedThreads), 0, s, B);
 }
 
 cudaError_t launch_reduce(const spmm_plan *p, int64_t n, void *Y, int64_t ldy, cudaStream_t s) {

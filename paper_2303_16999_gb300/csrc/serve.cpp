@@ -254,8 +254,8 @@ void serve_server::batcher_loop() {
             if (tc) {
                 e = launch_tc_batch(cnt, plans.data(), xs.data(), ns.data(), lxs.data(), ys.data(),
                                     lys.data(), s, false);
-                for (int i = 0; i < cnt && e == cudaSuccess; ++i)
-                    if (plans[i]->n_red > 0) e = launch_reduce(plans[i], ns[i], ys[i], lys[i], s);
+                if (e == cudaSuccess)
+                    e = launch_reduce_tc(cnt, plans.data(), ns.data(), ys.data(), lys.data(), s);
             } else {
                 spmm_status st = spmm_run(plans[0], nullptr, nullptr, nullptr, xs[0], ns[0],
                                           lxs[0], ys[0], lys[0], s);

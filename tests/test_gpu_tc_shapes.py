@@ -47,3 +47,36 @@ def test_joint_boxes_with_2d_maps(n, geo, ct):
     absent where it lies past n; k ends inside a box (31 tile columns)."""
     case = _problem(300 + n, 272, 496, n, 4, 68 * 124 // 2, torch.bfloat16)
     _run(*case, rows_per_group=16, stage_geometry=geo, col_tiles=ct)
+
+
+@pytest.mark.parametrize("n,pad", [(1, 0), (3, 1), (4, 0), (5, 3), (64, 4), (100, 2), (131, 0)])
+@pytest.mark.parametrize("splits", [2, 7, 8, 9, 20])
+def test_split_groups_reduction(n, pad, splits):
+    """The reduction of groups split along k: values a thread adds run over
+    row ends (n not a multiple of 4), rows of Y aligned and not, and more
+    partials than one pass of loads (8)."""
+    case = _problem(500 + n, 400, 1600, n, 8, 50 * 200 // 4, torch.float16)
+    info = _run(*case, pad=pad, rows_per_group=16, k_splits=splits)
+    assert info["n_reductions"] == 2 and info["n_items"] > 2 * (splits - 1)
+
+
+def test_batch_of_split_plans_one_reduction():
+    """Several split plans of one batch share a reduction launch (odd and even
+    n, padded Y); each equals its exact product."""
+    plans, xs, ys, wants = [], [], [], []
+    for i, n in enumerate((3, 40, 129, 64, 20)):
+        c, vals, x, want = _problem(700 + i, 320 + 16 * i, 2048, n, 8, (40 + 2 * i) * 64,
+                                    torch.bfloat16)
+        p = S.Plan(c["m"], c["k"], n, 8, w_dtype=S.BF16, brow=c["brow"], bcol=c["bcol"],
+                   kernel="tc", **({} if i == 3 else dict(rows_per_group=16, k_splits=3 + i)))
+        p.pack(vals)
+        plans.append(p)
+        xs.append(x)
+        ys.append(torch.full((c["m"], n + i), float("nan"), dtype=torch.bfloat16,
+                             device="cuda")[:, :n])
+        wants.append(want)
+    S.spmm_batch_run(plans, xs, ys)
+    torch.cuda.synchronize()
+    for p, y, want in zip(plans, ys, wants):
+        assert p.status() == 0 and torch.equal(y, want)
+        p.close()
