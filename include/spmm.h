@@ -109,7 +109,9 @@ typedef struct {
 /* Planner options; pass NULL for defaults (all fields 0). */
 typedef struct {
     int32_t kernel;               /* spmm_kernel */
-    int32_t rows_per_group;       /* TC: tile rows (16 rows each) per group, 1..16; 0 = planner's choice */
+    int32_t rows_per_group;       /* TC: tile rows (16 rows each) per group, 1..16; 0 = planner's choice
+                                     (static plans whose 16-row groups would not occupy the GPU: rows
+                                     per group and splits along k together) */
     int32_t max_per_item;         /* TC: entries per work item; GATHER: blocks per row item; 0 = planner's choice */
     int32_t host_only;            /* 1 = build the static plan on the host only (no device memory, no
                                      CUDA calls): for inspection with spmm_plan_get_array */
@@ -157,8 +159,9 @@ typedef struct {
     int32_t k_splits;             /* static TC plans: split every tile-row group's entries (its
                                      tile columns, i.e. its share of k) into about this many work
                                      items of near-equal length, whose FP32 partials the split-row
-                                     reduction sums in a fixed order; 0 = only groups well above the
-                                     mean length are split.  Overrides max_per_item.  0 .. 1024,
+                                     reduction sums in a fixed order; 0 = planner's choice (small
+                                     plans, see rows_per_group) and groups well above the mean
+                                     length.  Overrides max_per_item.  0 .. 1024,
                                      else SPMM_ERR_ARG. */
 } spmm_plan_opts;
 

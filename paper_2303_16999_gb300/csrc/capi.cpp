@@ -548,6 +548,7 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
         }
     }
     const int64_t mb = m / b, mt = m / kTile;
+    bool auto_split = false;
     try {
         if (mode == SPMM_STATIC) {
             st = validate_pattern(m, k, b, pattern->nnzb, pattern->brow, pattern->bcol);
@@ -589,26 +590,45 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
                         p->groups = (dense || o.col_tiles == 2) ? qw : qn;
                     }
                 }
+                int splits = o.k_splits;
                 if (p->groups > 0)
                     p->R = (int)((mt + p->groups - 1) / p->groups);
                 else
                     p->R = o.rows_per_group ? o.rows_per_group : default_R(mt, n_max, p->sm_count);
+                if (p->groups == 0 && !o.rows_per_group && !o.max_per_item && !o.k_splits &&
+                    (mt + kMaxGroupRows - 1) / kMaxGroupRows * ((n_max + kNTile - 1) / kNTile) <
+                        p->sm_count) {
+                    // (two column tiles per CTA: 16-bit weights, as for large n;
+                    // a col_tiles option leaves groups and splits as they are, so
+                    // results do not depend on it)
+                    const int ct = w_dtype == SPMM_E4M3 ? 1 : 0;
+                    const TcShape sh =
+                        choose_tc_shape(m, k, b, p->nnzb, pattern->brow, pattern->bcol,
+                                        std::max<int64_t>(n_max, 1), p->sm_count, ct, p->R);
+                    p->R = sh.rows;
+                    splits = sh.splits > 1 ? sh.splits : 0;
+                    auto_split = splits > 0;
+                    p->auto_wide = o.col_tiles == 0 && sh.col_tiles == 2;
+                }
                 if (o.max_per_item && !o.k_splits) {
                     p->C = o.max_per_item;
                 } else {
-                    HostPlan probe;
-                    build_tc_plan(m, k, b, p->nnzb, pattern->brow, pattern->bcol, p->R, 1 << 30,
-                                  false, false, probe, p->groups);
-                    const int64_t G = (int64_t)probe.grp_rows.size();
-                    const int64_t E = (int64_t)probe.ent_col.size();
-                    if (o.k_splits) {
-                        // about k_splits items per group of mean length
-                        const int64_t per = G ? (E + G * o.k_splits - 1) / (G * o.k_splits) : 1;
+                    const int64_t G = p->groups > 0 ? p->groups
+                                                    : (int64_t)group_partition(mt, p->R).size();
+                    const int64_t E = count_entries(m, k, b, p->nnzb, pattern->brow, pattern->bcol,
+                                                    p->R, p->groups);
+                    if (splits) {
+                        // about that many items per group of mean length
+                        const int64_t per = G ? (E + G * splits - 1) / (G * splits) : 1;
                         p->C = (int)std::max<int64_t>(1, per);
                     } else {
                         // entries per group if spread evenly, with headroom:
-                        // only groups well above the mean are split
-                        p->C = (int)std::max<int64_t>(16, G ? (5 * E + 4 * G - 1) / (4 * G) : 16);
+                        // only groups well above the mean are split (the
+                        // reduction's launch costs what about 50 entries do:
+                        // 4096 x 4096, b = 16, d = 1/8, n = 64 took 11.5 us
+                        // with its ten longest groups split, 8.9 without)
+                        p->C = (int)std::max<int64_t>(
+                            48, G ? std::max((5 * E + 4 * G - 1) / (4 * G), (E + G - 1) / G + 48) : 48);
                     }
                 }
                 build_tc_plan(m, k, b, p->nnzb, pattern->brow, pattern->bcol, p->R, p->C, true,
@@ -621,6 +641,9 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
             p->n_tiles = (int64_t)p->hp.tile_row.size();
             if (kernel == SPMM_KERNEL_TC && p->n_entries > 0)
                 p->tc_geo = tc_geometry((double)p->n_tiles / (double)p->n_entries);
+            // (E4M3 plans split along k take the sparse-tile stages: as fast alone,
+            // and a batch, which runs in one geometry, needs no second records)
+            if (w_dtype == SPMM_E4M3 && auto_split) p->tc_geo = 1;
             if (kernel == SPMM_KERNEL_TC && o.stage_geometry) p->tc_geo = o.stage_geometry - 1;
         } else {
             p->nnzb_max = nnzb_max;

@@ -954,7 +954,7 @@ __global__ void quantize_e4m3_kernel(const U *__restrict__ src, int64_t nnzb, in
 bool use_wide(const spmm_plan *p, int64_t n, int x3d) {
     if (p->col_tiles == 1 || p->mode != SPMM_STATIC || n <= kNTile) return false;
     // forced: any n > 128 (2-D X maps included) and E4M3 weights as well
-    if (p->col_tiles == 2) return true;
+    if (p->col_tiles == 2 || p->auto_wide) return true;
     if (!x3d || p->wdt == SPMM_E4M3) return false;
     const int64_t units = p->n_items * ((n + kNTile - 1) / kNTile);
     return p->tc_geo == 0 && 2 * units >= (int64_t)SPMM_TC_WIDE_MIN * p->sm_count;

@@ -5,6 +5,7 @@
 // decomposition; they are stated independently, in plain Python, by the
 // test oracle, and the two must agree bit for bit.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <numeric>
 #include <vector>
@@ -301,6 +302,129 @@ void build_tc_plan(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *bro
     std::vector<int64_t> grows(G);
     for (int64_t g = 0; g < G; ++g) grows[g] = (int64_t)hp.grp_rows[g] * kTile;
     finish_items(items, sort_items, grows, hp);
+}
+
+int64_t count_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
+                      const int32_t *bcol, int64_t R, int64_t groups) {
+    const int64_t mt = m / kTile, words = (k / kTile + 63) / 64;
+    const std::vector<int64_t> sizes =
+        groups > 0 ? near_equal_partition(mt, groups) : group_partition(mt, R);
+    std::vector<int64_t> base(mt, 0);   // first bitmap word of a tile row's group
+    int64_t t = 0;
+    for (size_t g = 0; g < sizes.size(); ++g)
+        for (int64_t i = 0; i < sizes[g]; ++i) base[t++] = (int64_t)g * words;
+    std::vector<uint64_t> bits(sizes.size() * words, 0);
+    for (int64_t p = 0; p < nnzb; ++p) {
+        const int64_t tc = (int64_t)bcol[p] * b / kTile;
+        bits[base[(int64_t)brow[p] * b / kTile] + tc / 64] |= 1ull << (tc % 64);
+    }
+    int64_t n = 0;
+    for (uint64_t w : bits) n += __builtin_popcountll(w);
+    return n;
+}
+
+// ------------------------------------------------------- launch shape -----
+// Static tensor-core plans whose 16-row groups alone do not occupy the GPU
+// (small n_max or few tile rows) need more units than groups x column tiles.
+// Two ways: groups of fewer tile rows, which re-read X (every group brings
+// the slabs of its own columns), or 16-row groups split along k, whose FP32
+// partials a second launch adds up.  Which is faster depends on the pattern:
+// this picks the tile rows per group, the splits and one or two column tiles
+// per CTA by a model of the launch, fitted to 1270 timed launches on a GB300
+// (59 products, m and k 256 to 16384, n 9 to 2000; rms error 11 %):
+//   time = 5.06 + max(bytes through L2 at 15.2 TB/s x imbalance of the SMs,
+//                     waves x (1.14 + 0.0805 per entry + 0.0045 per tile of a
+//                              unit, 1.32 times that over two column tiles),
+//                     0.029 per TMA box of an SM x imbalance)       [us]
+//          + for split groups 2.07 + partials written and read at 5.96 TB/s.
+// Another shape than the rows-per-group rule's has to promise 10 % less.  On
+// those products the pick takes 1.02 times the best shape's time on average
+// and 0.80 times the rule's: 4096 x 16384, b = 8, d = 1/8: n = 24 62.0 -> 23.4
+// us, n = 200 82.3 -> 39.7; 4096 x 4096, b = 4, d = 1/8, n = 100 48.1 -> 16.4.
+namespace {
+struct ShapeCost {
+    int64_t mt, kt, n;
+    double sms;
+    // E entries and S tile slots in all groups of R tile rows
+    double us(int64_t R, double E, double S, int ct, int64_t splits) const {
+        const int64_t G = (mt + R - 1) / R, ntn = (n + kNTile - 1) / kNTile;
+        const int64_t nt = (n + kNTile * ct - 1) / (kNTile * ct);
+        const double items = (double)(G * splits), slots = ct == 2 ? sms : 2 * sms;
+        const double units = items * (double)nt, waves = std::ceil(units / slots);
+        const double full = units <= 2 * sms || ct == 2 ? sms : 2 * sms;
+        const double imb = std::ceil(units / full) * full / units;
+        const double bytes = E * 32.0 * (double)n + (double)nt * S * kTileBytes16;
+        double boxes = E * (double)ntn * (n % 64 == 0 || n <= 64 ? 1 : 2);
+        if (E > 0.9 * (double)(G * kt)) boxes /= 4;   // mostly joint boxes
+        const double unit =
+            waves * (1.14 + (0.0805 * E + 0.0045 * S) / items * (ct == 2 ? 1.32 : 1));
+        double t = 5.06 + std::max({bytes / 15.2e6 * imb, unit, 0.029 * boxes / sms * imb});
+        if (splits > 1) t += 2.07 + (double)splits * (double)(mt * kTile) * (double)n * 8 / 5.96e6;
+        if (ct == 2) t *= 0.95;   // (the model is this much too hard on wide launches)
+        return t;
+    }
+};
+}  // namespace
+
+TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
+                        const int32_t *bcol, int64_t n, int sms, int ct_only, int default_rows) {
+    const int64_t mt = m / kTile, kt = k / kTile;
+    TcShape best{default_rows, 1, ct_only ? ct_only : 1};
+    if (nnzb == 0) return best;
+    // tile occupancy of a sample of 16-row bands: one row mask per column
+    const int64_t bands = (mt + kMaxGroupRows - 1) / kMaxGroupRows;
+    const int64_t step = std::max<int64_t>(1, bands * kt / 16384);
+    std::vector<uint16_t> mask(((bands + step - 1) / step) * kt, 0);
+    for (int64_t p = 0; p < nnzb; ++p) {
+        const int64_t tr = (int64_t)brow[p] * b / kTile, band = tr / kMaxGroupRows;
+        if (band % step == 0)
+            mask[band / step * kt + (int64_t)bcol[p] * b / kTile] |=
+                (uint16_t)(1u << (tr % kMaxGroupRows));
+    }
+    const ShapeCost cost{mt, kt, n, (double)sms};
+    const double scale = (double)bands / (double)((bands + step - 1) / step);
+    std::vector<int> rows;
+    std::vector<std::pair<int, int>> ivs;
+    double ref = 0, least = 0;
+    const int order[5] = {default_rows, 1, 2, 4, 8};
+    for (int i = 0; i < 6; ++i) {
+        const int R = i < 5 ? order[i] : kMaxGroupRows;
+        if (i > 0 && R == default_rows) continue;
+        // entries of R-row groups, and tile slots from every q-th of them
+        int64_t E = 0, sampled = 0, slots = 0;
+        const int64_t every = std::max<int64_t>(1, (int64_t)mask.size() / 512);
+        for (size_t c = 0; c < mask.size(); ++c)
+            for (int r0 = 0; r0 < kMaxGroupRows; r0 += R) {
+                const uint32_t g = (mask[c] >> r0) & ((1u << R) - 1);
+                if (!g) continue;
+                if (E++ % every) continue;
+                rows.clear();
+                for (int r = 0; r < R; ++r)
+                    if (g >> r & 1) rows.push_back(r);
+                cover_intervals(rows, ivs);
+                ++sampled;
+                for (const auto &iv : ivs) slots += iv.second;
+            }
+        const double e = (double)E * scale, s = sampled ? e * (double)slots / (double)sampled : 0;
+        const int64_t G = (mt + R - 1) / R;
+        for (int ct = 1; ct <= 2; ++ct) {
+            if ((ct_only && ct != ct_only) || (ct == 2 && (n <= kNTile || (!ct_only && n > 512))))
+                continue;
+            const int64_t nt = (n + kNTile * ct - 1) / (kNTile * ct);
+            const int64_t kmax = std::max<int64_t>(1, (ct == 2 ? sms : 2 * sms) / (G * nt));
+            for (int64_t q : {(int64_t)1, kmax / 3, kmax / 2, kmax * 2 / 3, kmax}) {
+                if (q < 1 || q > 1024 || q > std::max<int64_t>(1, kt / 4)) continue;
+                const double t = cost.us(R, e, s, ct, q);
+                if (ref == 0) ref = least = t;   // the default: first of all
+                // something else only for a clear gain over the default
+                if (t < least && t < 0.9 * ref) {
+                    least = t;
+                    best = TcShape{R, (int)q, ct};
+                }
+            }
+        }
+    }
+    return best;
 }
 
 }  // namespace spmm

@@ -73,6 +73,19 @@ void build_tc_plan(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *bro
                    const int32_t *bcol, int64_t R, int64_t C, bool sort_items, bool pad,
                    HostPlan &hp, int64_t groups = 0);
 
+// entries (distinct tile columns per tile-row group, summed) of a plan with
+// these groups
+int64_t count_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
+                      const int32_t *bcol, int64_t R, int64_t groups);
+// launch shape of a static tensor-core plan that 16-row groups alone would
+// not occupy the GPU with: tile rows per group, work items per group along k
+// and column tiles per CTA (ct_only: 0, or the only count allowed)
+struct TcShape {
+    int rows, splits, col_tiles;
+};
+TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
+                        const int32_t *bcol, int64_t n, int sms, int ct_only, int default_rows);
+
 // ------------------------------------------------------------------- plan
 // dynamic plans: scratch of the device re-partition
 struct DynBufs {
@@ -128,6 +141,7 @@ struct spmm_plan {
     int alt_geo = -1;
     int tc_geo = 0;                // TC stage geometry: 0 dense tiles, 1 sparse tiles
     int col_tiles = 0;             // TC: column tiles per CTA, 0 automatic (launch-time choice)
+    bool auto_wide = false;        // static TC, col_tiles 0: the planner chose two column tiles per CTA
     int64_t groups = 0;            // static TC: near-equal tile-row groups (0: equal partition by R)
     bool f32_blocks = false;       // FP32 b >= 4 plans AUTO chose: the block kernel (k_f32.cu),
                                    // values packed column by column within each block

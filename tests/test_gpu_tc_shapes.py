@@ -60,6 +60,20 @@ def test_split_groups_reduction(n, pad, splits):
     assert info["n_reductions"] == 2 and info["n_items"] > 2 * (splits - 1)
 
 
+@pytest.mark.parametrize("m,k,n,b,d,dt", [
+    (4096, 16384, 24, 8, 1 / 8, torch.bfloat16), (4096, 16384, 200, 8, 1 / 8, torch.float16),
+    (4096, 4096, 100, 4, 1 / 8, torch.bfloat16), (1024, 4096, 33, 8, 1 / 4, torch.float16),
+    (1024, 1024, 128, 8, 1 / 8, torch.bfloat16), (48, 8192, 300, 16, 1 / 2, torch.float16),
+    (16, 65536, 9, 16, 1.0, torch.bfloat16), (2048, 32, 64, 4, 1 / 2, torch.float16)])
+def test_planner_shapes_exact(m, k, n, b, d, dt):
+    """Plans whose shape the planner chooses, against the 64-bit product; a
+    col_tiles option changes neither groups nor splits."""
+    case = _problem(m + n, m, k, n, b, int((m // b) * (k // b) * d), dt)
+    infos = [_run(*case, col_tiles=ct) for ct in (0, 1, 2)]
+    for f in ("rows_per_group", "max_per_item", "n_items", "n_reductions"):
+        assert len({i[f] for i in infos}) == 1, f
+
+
 def test_batch_of_split_plans_one_reduction():
     """Several split plans of one batch share a reduction launch (odd and even
     n, padded Y); each equals its exact product."""
