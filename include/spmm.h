@@ -267,7 +267,7 @@ typedef struct {
     int32_t col_tiles;            /* TC: the col_tiles option the plan runs with (0, 1 or 2) */
     int32_t index_bytes;          /* bytes per column index the product reads: 2 for static
                                      GATHER plans with k <= 65536 (a 16-bit copy of col_idx,
-                                     read by the n <= 8 kernel that keeps X in shared memory),
+                                     read by the kernels that keep X in shared memory),
                                      else 4 */
 } spmm_plan_info;
 

@@ -192,6 +192,20 @@ static spmm_status upload_plan(spmm_plan *p) {
         // the b = 1 gather's column indices in half the bytes
         const std::vector<uint16_t> c16(hp.col_idx.begin(), hp.col_idx.end());
         e = upload(p, &p->d_col16, c16);
+        // where each part of k starts in every row
+        const int64_t pw = (p->k + kGxParts - 1) / kGxParts, m = p->m;
+        std::vector<int32_t> ptr(m * kGxParts + 1);
+        for (int64_t r = 0; r < m; ++r) {
+            int32_t i = hp.row_ptr[r];
+            for (int q = 0; q < kGxParts; ++q) {
+                ptr[r * kGxParts + q] = i;
+                i = (int32_t)(std::lower_bound(hp.col_idx.begin() + i,
+                                               hp.col_idx.begin() + hp.row_ptr[r + 1],
+                                               (q + 1) * pw) - hp.col_idx.begin());
+            }
+        }
+        ptr[m * kGxParts] = m ? hp.row_ptr[m] : 0;
+        if (e == cudaSuccess) e = upload(p, &p->d_gx_ptr, ptr);
     }
     if (p->kernel == SPMM_KERNEL_TC) {
         UP(d_grp_row0, grp_row0);
@@ -833,17 +847,22 @@ spmm_status spmm_pack_values(spmm_plan *plan, const void *d_values, const float 
 static spmm_status launch_product(spmm_plan *p, const void *d_X, int64_t n, int64_t ldx,
                                   void *d_Y, int64_t ldy, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
+    bool whole = false;   // the launch leaves no split rows to reduce
     switch (p->kernel) {
         case SPMM_KERNEL_PLAIN:
             e = p->f32_blocks ? launch_f32(p, d_X, n, ldx, d_Y, ldy, s)
                               : launch_plain(p, d_X, n, ldx, d_Y, ldy, s);
             break;
-        case SPMM_KERNEL_GATHER: e = launch_gather(p, d_X, n, ldx, d_Y, ldy, s); break;
+        case SPMM_KERNEL_GATHER:
+            whole = gather_xs_takes(p, n);
+            e = whole ? launch_gather_xs(p, d_X, n, ldx, d_Y, ldy, s)
+                      : launch_gather(p, d_X, n, ldx, d_Y, ldy, s);
+            break;
         case SPMM_KERNEL_TC: e = launch_tc(p, d_X, n, ldx, d_Y, ldy, s); break;
         case SPMM_KERNEL_BGATHER: e = launch_bgather(p, d_X, n, ldx, d_Y, ldy, s); break;
         default: set_error("bad kernel"); return SPMM_ERR_ARG;
     }
-    if (e == cudaSuccess && p->n_red > 0 && p->kernel != SPMM_KERNEL_PLAIN)
+    if (e == cudaSuccess && p->n_red > 0 && p->kernel != SPMM_KERNEL_PLAIN && !whole)
         e = p->kernel == SPMM_KERNEL_TC && p->mode == SPMM_STATIC
                 ? launch_reduce_tc(1, &p, &n, &d_Y, &ldy, s)
                 : launch_reduce(p, n, d_Y, ldy, s);

@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <atomic>
 
+#include "fma16.cuh"
 #include "pdl.cuh"
 #include "spmm_internal.h"
 
@@ -360,20 +361,17 @@ __global__ void __launch_bounds__(kG1Warps * 32, 1) gather1_kernel(
 #pragma unroll
             for (int e = 0; e < 8; ++e) x[e] = *reinterpret_cast<const Pack<T, V> *>(xs + cq[e] * V);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float wf = Vec<T>::to_f(w.v[e]);
+            for (int e = 0; e < 8; ++e)
 #pragma unroll
-                for (int v = 0; v < V; ++v) acc[v] = fmaf(wf, Vec<T>::to_f(x[e].v[v]), acc[v]);
-            }
+                for (int v = 0; v < V; ++v) acc[v] = fma16(w.v[e], x[e].v[v], acc[v]);
         } else {
             const int32_t p0 = m.base + 8 * lane;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 if (p0 + e >= m.beg && p0 + e < m.end) {
                     const Pack<T, V> x = *reinterpret_cast<const Pack<T, V> *>(xs + cq[e] * V);
-                    const float wf = Vec<T>::to_f(w.v[e]);
 #pragma unroll
-                    for (int v = 0; v < V; ++v) acc[v] = fmaf(wf, Vec<T>::to_f(x.v[v]), acc[v]);
+                    for (int v = 0; v < V; ++v) acc[v] = fma16(w.v[e], x.v[v], acc[v]);
                 }
             }
         }
@@ -438,14 +436,14 @@ __global__ void __launch_bounds__(512, SPMM_G1_BLOCKS) gather1g_kernel(
         float acc[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = 0.f;
-        auto add = [&](int32_t c, float w) {
+        auto add = [&](int32_t c, T w) {
             const Pack<T, V> x = *reinterpret_cast<const Pack<T, V> *>(xb + (int64_t)c * lx);
 #pragma unroll
-            for (int v = 0; v < V; ++v) acc[v] = fmaf(w, Vec<T>::to_f(x.v[v]), acc[v]);
+            for (int v = 0; v < V; ++v) acc[v] = fma16(w, x.v[v], acc[v]);
         };
         // head up to a multiple of 4 (vector alignment), one non-zero per lane
         const int32_t h = min(end, (beg + 3) & ~3);
-        if (beg + lane < h) add(col_idx[beg + lane], Vec<T>::to_f(vals[beg + lane]));
+        if (beg + lane < h) add(col_idx[beg + lane], vals[beg + lane]);
         // full passes: no bounds checks
         int32_t base = h;
         for (; base + 128 * kRounds <= end; base += 128 * kRounds) {
@@ -459,10 +457,10 @@ __global__ void __launch_bounds__(512, SPMM_G1_BLOCKS) gather1g_kernel(
             }
 #pragma unroll
             for (int q = 0; q < kRounds; ++q) {
-                add(c[q].x, Vec<T>::to_f(w[q].v[0]));
-                add(c[q].y, Vec<T>::to_f(w[q].v[1]));
-                add(c[q].z, Vec<T>::to_f(w[q].v[2]));
-                add(c[q].w, Vec<T>::to_f(w[q].v[3]));
+                add(c[q].x, w[q].v[0]);
+                add(c[q].y, w[q].v[1]);
+                add(c[q].z, w[q].v[2]);
+                add(c[q].w, w[q].v[3]);
             }
         }
         // the last partial pass
@@ -489,7 +487,7 @@ __global__ void __launch_bounds__(512, SPMM_G1_BLOCKS) gather1g_kernel(
                 const int32_t cq[4] = {c[q].x, c[q].y, c[q].z, c[q].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (i0 + e < end) add(cq[e], Vec<T>::to_f(w[q].v[e]));
+                    if (i0 + e < end) add(cq[e], w[q].v[e]);
             }
         }
 #pragma unroll
@@ -811,6 +809,11 @@ cudaError_t launch_plain(const spmm_plan *p, const void *X, int64_t n, int64_t l
     pdl_launch(plain_f32_kernel, dim3(grid), dim3(128), 0, s, p->d_row_ptr, p->d_col_idx,
         (const float *)p->d_packed, (const float *)X, ldx, (float *)Y, ldy, p->m, n, p->b);
     return cudaGetLastError();
+}
+
+bool gather_ring_fits(const spmm_plan *p, int64_t n) {
+    return p->xdt == SPMM_F32 ? p->k * n * 4 <= g1_x_budget<float, uint16_t, kG1Stages - 1>()
+                              : p->k * n * 2 <= g1_x_budget<__half, uint16_t, kG1Stages - 1>();
 }
 
 cudaError_t launch_gather(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, void *Y,

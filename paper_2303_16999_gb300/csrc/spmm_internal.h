@@ -16,6 +16,7 @@ constexpr int kTileBytes16 = 512;  // 16 x 16 16-bit tile in the MMA operand lay
 constexpr int kNTile = 128;        // n columns per tensor-core work unit (MMA M)
 constexpr int kMaxGroupRows = 16;  // tile rows per group: 2 x 16 x 16 TMEM columns = 512
 constexpr int kItemFields = 6;     // group/row, begin, end, chunk, n_chunks, ws_slot
+constexpr int kGxParts = 8;        // parts of k a row's non-zeros are split into (k_gather_xs.cu)
 constexpr int kDynMaxTileCols = 4096;  // dynamic TC plans: k <= 65536 (per-group smem bitmaps)
 
 // dynamic plans: device-side counters written by the re-partition
@@ -135,6 +136,7 @@ struct spmm_plan {
             *d_blk_off = nullptr, *d_grp_ebeg = nullptr;
     uint32_t *d_srec = nullptr, *d_sprog = nullptr;  // TC: stage records and MMA programs
     uint16_t *d_col16 = nullptr;   // static GATHER plans, k <= 65536: col_idx in 16 bits
+    int32_t *d_gx_ptr = nullptr;   // with it: the first non-zero of every (row, part of k)
     // TC, batched with plans of the other stage geometry: this plan's stage
     // records cut for that geometry (built on first use), geometry alt_geo
     uint32_t *d_srec_alt = nullptr, *d_sprog_alt = nullptr;
@@ -196,6 +198,12 @@ cudaError_t launch_pack_tiles(const spmm_plan *p, const void *d_values, const fl
                               const int32_t *d_nnzb, cudaStream_t s);
 cudaError_t launch_plain(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
                          int64_t ldy, cudaStream_t s);
+// whether X of n columns fits the gather ring kernel's shared memory
+bool gather_ring_fits(const spmm_plan *p, int64_t n);
+// b = 1 with X in shared memory (k_gather_xs.cu); whether it takes n columns
+bool gather_xs_takes(const spmm_plan *p, int64_t n);
+cudaError_t launch_gather_xs(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
+                             int64_t ldy, cudaStream_t s);
 // FP32 blocks, b >= 4 (k_f32.cu); launch_plain is the one-thread-per-output kernel
 cudaError_t launch_f32(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
                        int64_t ldy, cudaStream_t s);
