@@ -20,31 +20,33 @@
 // StageGeom::tiles W tiles, in one of two geometries the plan picks (dense
 // or sparse tiles).  How a work item's entries fall into stages, and the
 // MMAs of each stage (one word per MMA: slab, first W tile, first tile row,
-// rows), is fixed by the plan, so
+// rows; one list per half of the tile rows), is fixed by the plan, so
 // stage_build_kernel writes it once per plan (every call for dynamic plans)
 // as stage records.  Three producer warps follow the records with three in
 // flight: warp 0 copies the stage's W tiles (contiguous in the packed array,
 // one bulk copy) and its MMA program into shared memory, warps 6 and 7
 // request the two halves of its X slabs (one TMA per slab, both 64-column
 // halves in one 3-D box when n is a multiple of 64).  Issuing a copy costs
-// its warp a few hundred cycles, so they run side by side.  One lane of an
-// MMA warp walks the program words in order and issues every MMA of its
-// column tile, so the order of accumulation into every column is fixed.
-// With two stages the ring is bound by the copy latency (a stage is refilled
-// only after its MMAs complete).
+// its warp a few hundred cycles, so they run side by side.  Two MMA warps
+// (1: tile rows 0-7, 8: rows 8-15) stay converged: each lane loads one
+// program word and the warp walks them with one shuffle per MMA, issuing
+// through elect.sync; each owns its accumulator columns, so the order of
+// accumulation into every column is fixed.  With two stages the ring is
+// bound by the copy latency (a stage is refilled only after its MMAs
+// complete): each role spends about a third of a stage waiting.
 //
 // Wide launches (stage geometries 2 and 3): one CTA per SM covers two
 // 128-column tiles of n with all 512 TMEM columns; each stage holds both
 // tiles' X slabs and one set of W tiles, and every MMA word is issued once
-// per tile, so each W tile is read from L2 once per 256 columns.  One MMA
-// warp per column tile keeps the issue rate of two narrow CTAs.
+// per tile, so each W tile is read from L2 once per 256 columns.  Four MMA
+// warps (row half x column tile) keep the issue rate of two narrow CTAs.
 //
-// Warp roles (256 threads; wide: 288, wide sparse-tile: 352): warp 0 = W
-// producer, warp 1 = MMA issuer (owns TMEM; wide: 8 issues the second column
-// tile's MMAs), warps 2..5 = epilogue (TMEM -> registers -> Y or workspace)
-// and, for E4M3 weights, converters, warps 6 and 7 = X producers (wide: one
-// column tile each; wide sparse-tile: warps 9 and 10 take a share of each
-// tile's slabs).
+// Warp roles (288 threads; wide: 352, wide sparse-tile: 416): warp 0 = W
+// producer, warps 1 and 8 = MMA issuers (warp 1 owns TMEM; wide: 9 and 10
+// issue the second column tile's MMAs), warps 2..5 = epilogue (TMEM ->
+// registers -> Y or workspace) and, for E4M3 weights, converters, warps 6
+// and 7 = X producers (wide: one column tile each; wide sparse-tile: warps
+// 11 and 12 take a share of each tile's slabs).
 // Every mbarrier wait is bounded (globaltimer); on expiry the CTA records
 // SPMM_ERR_TIMEOUT in the plan's status word, stops, frees TMEM and exits.
 #include <cuda.h>
@@ -142,8 +144,6 @@ constexpr int kRowCap = SPMM_TC_RCAP;
 constexpr int kAccCols = kRowCap * kTile;                         // TMEM columns per buffer
 constexpr int kMaxBatch = 64;                                     // problems per launch
 
-constexpr int tc_threads(int geo) { return geo == 3 ? 352 : geo == 2 ? 288 : 256; }
-
 // Stage layout: X slabs (of each column tile the CTA covers) | 16-bit W
 // tiles (MMA B operand) | (E4M3 only) the FP8 codes and their scales as
 // loaded, which the converter warps expand into the 16-bit area.
@@ -157,8 +157,8 @@ template <bool W8, int GEO> struct StageGeom {
     // carry up to 2 x 8 separate slab copies, so two warps share each tile's
     static constexpr int xprod = GEO == 3 ? 2 : 1;
     static constexpr int producers = sets > 1 ? 1 + sets * xprod : 3;   // W + X warps
-    static constexpr int threads = tc_threads(GEO);
-    static constexpr int mma_warps = sets;          // one per column tile
+    static constexpr int threads = GEO == 3 ? 416 : sets > 1 ? 352 : 288;
+    static constexpr int mma_warps = 2 * sets;      // one per row half and column tile
     // E4M3 weights: the same stage shapes whether a CTA covers one column
     // tile or two (its W tiles, codes and scales serve both)
     static constexpr int stages = W8 ? (base ? SPMM_TC_STAGES8_S : SPMM_TC_STAGES8)
@@ -191,31 +191,35 @@ constexpr int kAccBufs = SPMM_TC_ACCBUFS;
 static_assert(kAccBufs * SPMM_TC_CTAS * SPMM_TC_RCAP * 16 <= 512, "TMEM columns per SM");
 constexpr int kCtasPerSm = SPMM_TC_CTAS;
 static_assert(kRowCap <= kMaxGroupRows && kRowCap <= 16, "a stage must hold a full entry");
-constexpr int kMmaWarpsMax = 2;
+constexpr int kThreads = 288;                                     // one column tile per CTA
+constexpr int kMmaWarpsMax = 4;
 constexpr int kXWarp0 = 6, kXWarp1 = 7;                           // X-slab producers (two halves)
-constexpr int kMmaWarp1 = 8;                                      // wide: MMAs of the second column tile
-constexpr int kXWarp2 = 9;                                        // wide sparse: warps 9, 10 as well
+constexpr int kXWarp2 = 11;                                       // wide sparse: warps 11, 12 as well
+constexpr int kMmaWarpHi = 8;                                     // MMAs of tile rows 8-15
 constexpr int kProducersMax = 5;                                  // W + up to four X
 constexpr unsigned long long kWaitNs = 2000000000ull;             // 2 s: default per wait, and
                                                                   // every wait of the abort drain
 
 // A stage's MMA program: one word per MMA (slab index in the stage | first
 // W tile in the stage << 4 | first tile row << 12 | rows << 16), so the MMA
-// warps decode nothing on their critical path.
+// warps decode nothing on their critical path.  Two MMA warps split the
+// accumulator by tile rows (0-7 and 8-15; an interval crossing row 8 becomes
+// two MMAs), so each TMEM column is written by one warp in a fixed order.
 // (StageGeom checks that a stage record's 12 X columns suffice)
 // Stage record (built before the launch; a work item's stages are records
 // e0, e0 + 1, ... where e0 is its first entry, since every stage holds at
-// least one entry): info (MMAs | entries << 12
-// | last << 31), W tiles, first W tile, the X column of each entry; the
-// stage's MMA program lives in a parallel array of kMmaStage words per record.
-struct __align__(16) StageMeta {
-    uint32_t prog[kMmaStage];      // MMA words
+// least one entry): info (MMAs of rows 0-7 | MMAs of rows 8-15 << 6 |
+// entries << 12 | last << 31), W tiles, first W tile, the X column of each
+// entry; the stage's MMA program lives in a parallel array of 2 x kMmaStage
+// words per record, (rows 0-7 word, rows 8-15 word) pairs.
+struct StageMeta {
     uint32_t info;                 // as in the stage record
     uint32_t nslots;               // W tiles in the stage
+    uint32_t prog[2][kMmaStage];   // MMA words of rows 0-7 and of rows 8-15
 };
 
 // Control block after the stages; S = the geometry's stage count.
-template <int S> struct __align__(16) SmemT {
+template <int S> struct __align__(8) SmemT {
     uint64_t full[S], empty[S], conv[S], accf[kAccBufs], acce[kAccBufs];
     uint64_t drain;                // abort: one tcgen05.commit per MMA warp
     uint64_t never;                // failure-detection tests: nothing arrives here
@@ -329,7 +333,7 @@ __device__ __forceinline__ Unit decode_unit(const TcBatch &B, int64_t u) {
 }
 
 template <typename T, bool W8, int GEO>
-__global__ void __launch_bounds__(tc_threads(GEO), GEO >= 2 ? 1 : kCtasPerSm)
+__global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GEO >= 2 ? 1 : kCtasPerSm)
     tc_kernel(const __grid_constant__ TcBatch B) {
     pdl_enter();
     using G = StageGeom<W8, GEO>;
@@ -412,13 +416,13 @@ __global__ void __launch_bounds__(tc_threads(GEO), GEO >= 2 ? 1 : kCtasPerSm)
             const int n0 = un.t * kNTile * G::sets;
             // wide: the second column tile, unless it lies wholly past n
             const bool two = G::sets > 1 && n0 + kNTile < P.n;
-            // lane l: word (l & 15) of the record, and (W producer) program words 2l, 2l + 1
+            // lane l: word (l & 7) of the record, and (W producer) program word l
             auto ld_rec = [&](int32_t r) -> uint32_t {
                 return r < e1 ? __ldg(P.srec + (int64_t)r * kRecWords + (lane & (kRecWords - 1))) : 0u;
             };
             auto ld_prog = [&](int32_t r) -> uint2 {
                 return (wprod && r < e1)
-                           ? __ldg((const uint2 *)(P.sprog + (int64_t)r * kMmaStage) + lane)
+                           ? __ldg((const uint2 *)(P.sprog + (int64_t)r * 2 * kMmaStage) + lane)
                            : make_uint2(0u, 0u);
             };
             // one stage from its record word (lane l: word l & 7) and program
@@ -438,7 +442,8 @@ __global__ void __launch_bounds__(tc_threads(GEO), GEO >= 2 ? 1 : kCtasPerSm)
                 if (!__shfl_sync(0xffffffffu, w, 0)) return -1;
                 uint8_t *st = stages + stage * G::bytes;
                 if (wprod) {
-                    ((uint2 *)sm->meta[stage].prog)[lane] = pc;
+                    sm->meta[stage].prog[0][lane] = pc.x;
+                    sm->meta[stage].prog[1][lane] = pc.y;
                     if (lane == 0) {
                         sm->meta[stage].info = info;
                         sm->meta[stage].nslots = nslots;
@@ -585,102 +590,91 @@ __global__ void __launch_bounds__(tc_threads(GEO), GEO >= 2 ? 1 : kCtasPerSm)
             sm->abort_flag = 1;
         }
         if (lane == 0) sm->issued[pid] = issued;
-    } else if (warp == 1 || warp == kMmaWarp1) {
-        // ------------------------- MMA issuers (one elected lane per warp)
-        // warp 1: the first column tile; wide CTAs, warp 8: the second.  One
-        // lane runs the whole role: the MMA warp is what a stage waits for
-        // (timed inside the launch, 4096 x 4096, b = 4, d = 1/8, n = 1000:
-        // 916 cycles per stage, of them 590 in issuing five MMAs, each behind
-        // a shuffle and an election, against 600 with the MMAs left out), so
-        // it reads four program words at once and decodes them side by side.
-        // One lane now issues fast enough for a CTA, so an interval of tile
-        // rows is one MMA whatever its length (two warps used to issue the
-        // halves above and below row 8, with A read twice).  4096 x 4096,
-        // n = 2048: b = 8, d = 1/4 51.0 -> 47.1 us, d = 1/16 38.0 -> 36.2;
-        // b = 4, d = 1/8, n = 2000 56.7 -> 49.1.
-        const int tset = warp == 1 ? 0 : 1;   // column tile
+    } else if (warp == 1 || (warp >= kMmaWarpHi && warp <= kMmaWarpHi + 2)) {
+        // ------------------------------- MMA issuers (converged warps)
+        // warps 1 / 8: tile rows 0-7 / 8-15 of the first column tile; wide
+        // CTAs: warps 9 / 10 the same rows of the second column tile
+        const int mw = warp == 1 ? 0 : warp - kMmaWarpHi + 1;   // 0..3
+        const int half = mw & 1;              // tile rows 0-7 / 8-15
+        const int tset = mw >> 1;             // column tile
         constexpr uint32_t idesc0 = make_idesc(Cvt<T>::fmt, kNTile, 0);
-        if (elect_one()) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int32_t consumed = 0;
-            bool ok = true;
-            int local = 0;
-            for (int64_t u = blockIdx.x; u < nunits; u += gridDim.x, ++local) {
-                const Unit un = decode_unit(B, u);
-                const int32_t *it = B.prob[un.p].items + un.item * kItemFields;
-                const bool has_entries = it[2] > it[1];
-                const bool two =
-                    G::sets > 1 && (int64_t)un.t * kNTile * G::sets + kNTile < B.prob[un.p].n;
-                const int ab = local % kBufs;
-                const uint32_t aphase = (local / kBufs) & 1;
-                ok = mbar_wait(&sm->acce[ab], aphase ^ 1, sm, B.wait_ns);
+        int stage = 0;
+        uint32_t phase = 0;
+        int32_t consumed = 0;
+        bool ok = true;
+        int local = 0;
+        for (int64_t u = blockIdx.x; u < nunits; u += gridDim.x, ++local) {
+            const Unit un = decode_unit(B, u);
+            const int32_t *it = B.prob[un.p].items + un.item * kItemFields;
+            const bool has_entries = it[2] > it[1];
+            const bool two = G::sets > 1 && (int64_t)un.t * kNTile * G::sets + kNTile < B.prob[un.p].n;
+            const int ab = local % kBufs;
+            const uint32_t aphase = (local / kBufs) & 1;
+            int w = 1;
+            if (lane == 0) w = mbar_wait(&sm->acce[ab], aphase ^ 1, sm, B.wait_ns) ? 1 : 0;
+            ok = __shfl_sync(0xffffffffu, w, 0) != 0;
+            tc_fence_after();
+            const uint32_t dbase = tmem + ab * G::sets * kAccCols;
+            bool last = !has_entries;
+            while (ok && !last) {
+                if (lane == 0)
+                    w = mbar_wait(W8 ? &sm->conv[stage] : &sm->full[stage], phase, sm, B.wait_ns) ? 1 : 0;
+                if (!__shfl_sync(0xffffffffu, w, 0)) {
+                    ok = false;
+                    break;
+                }
+                __syncwarp();   // orders lane 0's acquire before every lane's reads
                 tc_fence_after();
-                // wide, second column tile: the same W tiles against that
-                // tile's slabs, into the second accumulator set
-                const uint32_t dbase = tmem + (ab * G::sets + tset) * kAccCols;
-                bool last = !has_entries;
-                while (ok && !last) {
-                    if (!mbar_wait(W8 ? &sm->conv[stage] : &sm->full[stage], phase, sm, B.wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    ++consumed;
-                    const uint32_t info = sm->meta[stage].info;
-                    // (a second column tile wholly past n gets no MMAs)
-                    const int nmma = (tset && !two) ? 0 : (int)(info & 127u);
-                    last = (info >> 31) != 0;
-                    const uint32_t sbase = smem_u32(stages + stage * G::bytes);
-                    const bool joint = (info & kJointBit) != 0;
-                    const uint64_t adesc0 =
-                        (joint ? a_desc_joint(sbase) : a_desc(sbase)) + tset * (G::xset >> 4);
-                    const uint32_t astep = joint ? (kSlabBytes / 2) >> 4 : kSlabBytes >> 4;
-                    const uint64_t bdesc0 = b_desc(sbase + G::w16);
-                    auto issue = [&](uint32_t wd) {
-                        const uint32_t slab = wd & 15u, toff = (wd >> 4) & 255u;
-                        const uint32_t r0 = (wd >> 12) & 15u, len = (wd >> 16) & 31u;
-                        // descriptor start addresses are in 16-byte units (bits 0-13)
-                        tc_mma_acc(dbase + r0 * kTile, adesc0 + slab * astep,
-                                   bdesc0 + toff * (kTileBytes16 >> 4),
-                                   idesc0 | ((len * kTile) >> 3) << 17);
-                    };
-                    const uint4 *prog = (const uint4 *)sm->meta[stage].prog;
-                    int i = 0;
-                    for (; i + 4 <= nmma; i += 4) {
-                        const uint4 wd = prog[i >> 2];
-                        issue(wd.x);
-                        issue(wd.y);
-                        issue(wd.z);
-                        issue(wd.w);
-                    }
-                    if (i < nmma) {   // (words past nmma are unused)
-                        const uint4 wd = prog[i >> 2];
-                        issue(wd.x);
-                        if (i + 1 < nmma) issue(wd.y);
-                        if (i + 2 < nmma) issue(wd.z);
-                    }
-                    tc_commit(&sm->empty[stage]);
-                    if (++stage == kStages) {
-                        stage = 0;
-                        phase ^= 1;
-                    }
+                ++consumed;
+                // every lane reads the stage header and one program word
+                const uint32_t info = sm->meta[stage].info;
+                // (a second column tile wholly past n gets no MMAs)
+                const int nmma = (tset && !two) ? 0 : (int)((info >> (6 * half)) & 63u);
+                last = (info >> 31) != 0;
+                const uint32_t myword = sm->meta[stage].prog[half][lane];   // words >= nmma unused
+                const uint32_t sbase = smem_u32(stages + stage * G::bytes);
+                const bool joint = (info & kJointBit) != 0;
+                const uint64_t adesc0 = joint ? a_desc_joint(sbase) : a_desc(sbase);
+                const uint32_t astep = joint ? (kSlabBytes / 2) >> 4 : kSlabBytes >> 4;
+                const uint64_t bdesc0 = b_desc(sbase + G::w16);
+                for (int i = 0; i < nmma; ++i) {
+                    const uint32_t wd = __shfl_sync(0xffffffffu, myword, i);
+                    const uint32_t slab = wd & 15u, toff = (wd >> 4) & 255u;
+                    const uint32_t r0 = (wd >> 12) & 15u, len = (wd >> 16) & 31u;
+                    // descriptor start addresses are in 16-byte units (bits 0-13)
+                    // wide, second column tile: the same W tiles against that
+                    // tile's slabs, into the second accumulator set
+                    tc_mma_elect(dbase + tset * kAccCols + r0 * kTile,
+                                 adesc0 + tset * (G::xset >> 4) + slab * astep,
+                                 bdesc0 + toff * (kTileBytes16 >> 4),
+                                 idesc0 | ((len * kTile) >> 3) << 17, 1u);
+                }
+                if (lane == 0) tc_commit(&sm->empty[stage]);
+                __syncwarp();
+                if (++stage == kStages) {
+                    stage = 0;
+                    phase ^= 1;
+                }
+                if (B.stall) {
                     // failure-detection tests: a wait that nothing ends
-                    if (B.stall && !mbar_wait(&sm->never, 0, sm, B.wait_ns)) {
+                    if (lane == 0) w = mbar_wait(&sm->never, 0, sm, B.wait_ns) ? 1 : 0;
+                    if (!__shfl_sync(0xffffffffu, w, 0)) {
                         ok = false;
                         break;
                     }
                 }
-                if (!ok) break;
-                tc_commit(&sm->accf[ab]);
             }
+            if (!ok) break;
+            if (lane == 0) tc_commit(&sm->accf[ab]);
+            __syncwarp();
+        }
+        if (lane == 0) {
             if (!ok) {
                 record(B.status, kDevTimeout);
                 sm->abort_flag = 1;
             }
-            sm->consumed[tset] = consumed;
+            sm->consumed[mw] = consumed;
         }
-        __syncwarp();
     } else {
         // ------------------------- converters (E4M3) and epilogue
         const int q = warp & 3;              // TMEM lane quarter of this warp
@@ -858,8 +852,8 @@ __global__ void __launch_bounds__(tc_threads(GEO), GEO >= 2 ? 1 : kCtasPerSm)
         }
         // each MMA warp's issuing lane commits once more: the drain barrier
         // completes when every MMA any of them issued has completed
-        const bool mma_warp = warp == 1 || (G::sets > 1 && warp == kMmaWarp1);
-        if (mma_warp && elect_one()) tc_commit(&sm->drain);
+        const bool mma_warp = warp == 1 || (warp >= kMmaWarpHi && warp < kMmaWarpHi + G::mma_warps - 1);
+        if (mma_warp && lane == 0) tc_commit(&sm->drain);
         __syncthreads();
         if (threadIdx.x == 0) {
             const unsigned long long t0 = gtimer();
@@ -1135,14 +1129,14 @@ cudaError_t ensure_alt_records(spmm_plan *p, int geo, cudaStream_t s) {
     if (!p->d_srec_alt) {
         void *a = nullptr, *b = nullptr;
         cudaError_t e = cudaMalloc(&a, (size_t)E * kRecWords * sizeof(uint32_t));
-        if (e == cudaSuccess) e = cudaMalloc(&b, (size_t)E * kMmaStage * sizeof(uint32_t));
+        if (e == cudaSuccess) e = cudaMalloc(&b, (size_t)E * 2 * kMmaStage * sizeof(uint32_t));
         if (e != cudaSuccess) {
             if (a) cudaFree(a);
             return e;
         }
         p->allocations.push_back(a);
         p->allocations.push_back(b);
-        p->device_bytes += E * (kRecWords + kMmaStage) * (int64_t)sizeof(uint32_t);
+        p->device_bytes += E * (kRecWords + 2 * kMmaStage) * (int64_t)sizeof(uint32_t);
         p->d_srec_alt = (uint32_t *)a;
         p->d_sprog_alt = (uint32_t *)b;
     }
@@ -1262,7 +1256,7 @@ cudaError_t launch_stage_build(const spmm_plan *p, cudaStream_t s) {
 
 int64_t stage_record_words() { return kRecWords; }
 int tc_geometry(double tiles_per_entry) { return tiles_per_entry >= 8.0 ? 0 : 1; }
-int64_t stage_prog_words() { return kMmaStage; }
+int64_t stage_prog_words() { return 2 * kMmaStage; }
 
 cudaError_t launch_pack_tiles(const spmm_plan *p, const void *d_values, const float *d_scales,
                               const int32_t *d_nnzb, cudaStream_t s) {

@@ -120,20 +120,6 @@ __device__ __forceinline__ void mbar_arrive_tx(uint64_t *b, uint32_t bytes) {
                  : "memory");
 }
 
-// True in one lane of a converged warp (the same lane every time).
-__device__ __forceinline__ bool elect_one() {
-    uint32_t e;
-    asm volatile(
-        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n selp.u32 %0, 1, 0, e;\n}" : "=r"(e));
-    return e != 0;
-}
-// One accumulating MMA, issued by the calling thread.
-__device__ __forceinline__ void tc_mma_acc(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.eq.u32 p, 0, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc));
-}
 // One MMA issued by a single elected lane of a converged warp.
 __device__ __forceinline__ void tc_mma_elect(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                              uint32_t acc) {

@@ -17,7 +17,7 @@ namespace spmm {
 namespace {
 
 constexpr int kRecWords = 16;           // words per stage record
-constexpr int kMmaStage = 64;           // MMAs per stage (two program words per lane)
+constexpr int kMmaStage = 32;           // MMAs per stage and row half (one per lane)
 constexpr int kJointSlabs = 4;          // slabs of a joint X box
 // A stage whose entries are 2 to 4 consecutive tile columns (record info
 // bit 20) gets its X slabs in one TMA box of kJointSlabs slabs (with a 2-D X
@@ -30,12 +30,12 @@ constexpr int kBuildWarps = 16;         // warps of a stage_build_kernel CTA
 // independently: one CTA per work item, one warp per batch.  A warp cuts
 // its batch exactly as the producers consume it (consecutive entries while
 // the stage holds at most `ent_cap` X slabs, `tiles_cap` W tiles and
-// kMmaStage MMAs; one entry always fits), counts its stages,
+// kMmaStage MMAs per row half; one entry always fits), counts its stages,
 // and after a CTA-wide prefix of the counts writes its records at
 // e0 + (stages of earlier batches) + i, expanding every entry's row
 // intervals (runs of covered rows cut at interval starts) into MMA words:
-// slab | first W tile in the stage << 4 | first tile row << 12 | rows << 16.
-// Dynamic
+// slab | first W tile in the stage << 4 | first tile row << 12 | rows << 16,
+// one list per row half (an interval across row 8 is cut there).  Dynamic
 // plans read the item count and the status word on the device (a rejected
 // pattern builds nothing).
 
@@ -45,8 +45,8 @@ constexpr int kBuildWarps = 16;         // warps of a stage_build_kernel CTA
 struct BatchCut {
     int32_t mcol, mtb;      // entry's tile column and first tile
     uint32_t mcov;          // covered rows | interval starts << 16
-    int S, L;               // inclusive prefixes: tiles, MMAs
-    int nmma, mslots;       // this entry's MMAs (row intervals) and tiles
+    int S, L, H;            // inclusive prefixes: tiles, MMAs of each half
+    int nlo, nhi, mslots;   // this entry's MMAs per half and tiles
     int my_j, my_stage;     // start lane and index of this entry's stage
     int kst;                // lane k: start lane of stage k
     int cnt, nst;           // entries in the batch, stages
@@ -63,21 +63,37 @@ __device__ BatchCut cut_batch(int32_t eb, int32_t e1, int ent_cap, int tiles_cap
     c.mtb = valid ? ent_tbeg[e] : 0;
     c.mcov = valid ? (uint32_t)ent_cover[e] : 0u;
     const uint32_t cov = c.mcov & 0xFFFFu;
-    c.nmma = __popc(c.mcov >> 16);   // one per interval start
+    // this entry's MMAs per row half: intervals below / above row 8, an
+    // interval across it counting in both
+    int nlo = 0, nhi = 0;
+    for (uint32_t st = c.mcov >> 16; st; st &= st - 1) {
+        const uint32_t r0 = __ffs(st) - 1;
+        const uint32_t rest = st & (st - 1);
+        const uint32_t next = rest ? (uint32_t)(__ffs(rest) - 1) : 16u;
+        uint32_t len = (uint32_t)__ffs(~(cov >> r0)) - 1;   // run of covered rows
+        len = len < next - r0 ? len : next - r0;
+        nlo += r0 < 8;
+        nhi += r0 + len > 8;
+    }
+    c.nlo = nlo;
+    c.nhi = nhi;
     c.mslots = __popc(cov);
-    // inclusive prefix sums over the batch: tiles, MMAs
-    int S = c.mslots, L = c.nmma;
+    // inclusive prefix sums over the batch: tiles, MMAs of each half
+    int S = c.mslots, L = nlo, H = nhi;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int s2 = __shfl_up_sync(0xffffffffu, S, o);
         const int l2 = __shfl_up_sync(0xffffffffu, L, o);
+        const int h2 = __shfl_up_sync(0xffffffffu, H, o);
         if (lane >= o) {
             S += s2;
             L += l2;
+            H += h2;
         }
     }
     c.S = S;
     c.L = L;
+    c.H = H;
     c.cnt = min(32, e1 - eb);
     c.my_j = 0;
     c.my_stage = 0;
@@ -87,8 +103,9 @@ __device__ BatchCut cut_batch(int32_t eb, int32_t e1, int ent_cap, int tiles_cap
         // sums are monotone: the fitting lanes are contiguous from j
         const int Sb = j ? __shfl_sync(0xffffffffu, S, j - 1) : 0;
         const int Lb = j ? __shfl_sync(0xffffffffu, L, j - 1) : 0;
+        const int Hb = j ? __shfl_sync(0xffffffffu, H, j - 1) : 0;
         const bool fits = lane >= j && lane < j + ent_cap && lane < c.cnt &&
-                          S - Sb <= tiles_cap && L - Lb <= kMmaStage;
+                          S - Sb <= tiles_cap && L - Lb <= kMmaStage && H - Hb <= kMmaStage;
         const int nent = __popc(__ballot_sync(0xffffffffu, fits));
         if (lane >= j && lane < j + nent) {
             c.my_j = j;
@@ -104,7 +121,8 @@ __device__ BatchCut cut_batch(int32_t eb, int32_t e1, int ent_cap, int tiles_cap
 // The write pass of a cut batch, every stage at once: stores its records
 // from record index `rec`, expanding every entry's row intervals (runs of
 // covered rows cut at interval starts) into MMA words: slab | first W tile
-// in the stage << 4 | first tile row << 12 | rows << 16.
+// in the stage << 4 | first tile row << 12 | rows << 16, one list per row
+// half (an interval across row 8 is cut there).
 __device__ void write_batch(const BatchCut &c, bool last_batch, int32_t rec, uint32_t *srec,
                             uint32_t *sprog) {
     const int lane = threadIdx.x & 31;
@@ -113,27 +131,36 @@ __device__ void write_batch(const BatchCut &c, bool last_batch, int32_t rec, uin
     const int src = in && c.my_j > 0 ? c.my_j - 1 : 0;
     const int Sp = __shfl_sync(0xffffffffu, c.S, src);
     const int Lp = __shfl_sync(0xffffffffu, c.L, src);
+    const int Hp = __shfl_sync(0xffffffffu, c.H, src);
     if (in) {
         const bool first = c.my_j == 0;
-        uint32_t kw = (uint32_t)(c.L - c.nmma - (first ? 0 : Lp));
+        uint32_t klo = (uint32_t)(c.L - c.nlo - (first ? 0 : Lp));
+        uint32_t khi = (uint32_t)(c.H - c.nhi - (first ? 0 : Hp));
         uint32_t toff = (uint32_t)(c.S - c.mslots - (first ? 0 : Sp));
         const uint32_t slab = (uint32_t)(lane - c.my_j);
         const uint32_t cov = c.mcov & 0xFFFFu;
-        uint32_t *pr = sprog + (int64_t)(rec + c.my_stage) * kMmaStage;
+        uint32_t *pr = sprog + (int64_t)(rec + c.my_stage) * 2 * kMmaStage;
         for (uint32_t st = c.mcov >> 16; st; st &= st - 1) {
             const uint32_t r0 = __ffs(st) - 1;
             const uint32_t rest = st & (st - 1);
             const uint32_t next = rest ? (uint32_t)(__ffs(rest) - 1) : 16u;
             uint32_t len = (uint32_t)__ffs(~(cov >> r0)) - 1;
             len = len < next - r0 ? len : next - r0;
-            pr[kw++] = slab | toff << 4 | r0 << 12 | len << 16;
+            if (r0 < 8) {
+                const uint32_t l0 = r0 + len > 8 ? 8 - r0 : len;
+                pr[2 * klo++] = slab | toff << 4 | r0 << 12 | l0 << 16;
+            }
+            if (r0 + len > 8) {
+                const uint32_t a = r0 < 8 ? 8u : r0;   // first row at or above 8
+                pr[2 * khi++ + 1] = slab | (toff + (a - r0)) << 4 | a << 12 | (r0 + len - a) << 16;
+            }
             toff += len;
         }
     }
     // bit i: entry i is not one tile column past entry i - 1
     const int32_t pcol = __shfl_up_sync(0xffffffffu, c.mcol, 1);
     const uint32_t brk = __ballot_sync(0xffffffffu, lane > 0 && c.mcol != pcol + 1);
-    // records, kRecWords words per stage: word 0 the MMA count, entry
+    // records, kRecWords words per stage: word 0 the MMA counts, entry
     // count and flags, 1 the stage's tiles, 2 its first tile, 3 + i the X
     // column of its entry i
     for (int w0 = 0; w0 < c.nst * kRecWords; w0 += 32) {
@@ -145,18 +172,20 @@ __device__ void write_batch(const BatchCut &c, bool last_batch, int32_t rec, uin
         const int nent = jn - j;
         const int Se = __shfl_sync(0xffffffffu, c.S, jn - 1);
         const int Le = __shfl_sync(0xffffffffu, c.L, jn - 1);
+        const int He = __shfl_sync(0xffffffffu, c.H, jn - 1);
         const int Sb0 = __shfl_sync(0xffffffffu, c.S, max(j - 1, 0));
         const int Lb0 = __shfl_sync(0xffffffffu, c.L, max(j - 1, 0));
+        const int Hb0 = __shfl_sync(0xffffffffu, c.H, max(j - 1, 0));
         const int32_t stb = __shfl_sync(0xffffffffu, c.mtb, j);
         const int32_t xc = __shfl_sync(0xffffffffu, c.mcol, min(j + max(i - 3, 0), 31));
         if (w < c.nst * kRecWords) {
-            const int Sb = j ? Sb0 : 0, Lb = j ? Lb0 : 0;
+            const int Sb = j ? Sb0 : 0, Lb = j ? Lb0 : 0, Hb = j ? Hb0 : 0;
             const bool joint = nent >= 2 && nent <= kJointSlabs &&
                                ((brk >> (j + 1)) & ((1u << (nent - 1)) - 1u)) == 0;
             const bool last = last_batch && jn == c.cnt;
             uint32_t v = 0;
             if (i == 0)
-                v = (uint32_t)(Le - Lb) | (uint32_t)nent << 12 |
+                v = (uint32_t)(Le - Lb) | (uint32_t)(He - Hb) << 6 | (uint32_t)nent << 12 |
                     (joint ? kJointBit : 0u) | (last ? 0x80000000u : 0u);
             else if (i == 1) v = (uint32_t)(Se - Sb);
             else if (i == 2) v = (uint32_t)stb;

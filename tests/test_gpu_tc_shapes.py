@@ -94,29 +94,3 @@ def test_batch_of_split_plans_one_reduction():
     for p, y, want in zip(plans, ys, wants):
         assert p.status() == 0 and torch.equal(y, want)
         p.close()
-
-
-@pytest.mark.parametrize("geo", [1, 2])
-@pytest.mark.parametrize("rows", [(0, 16, 2), (1, 16, 2), (0, 16, 1), (7, 9, 1), (0, 8, 1)])
-def test_row_intervals_of_a_stage(geo, rows):
-    """Dynamic plans keep a group's gaps, so alternate tile rows make one MMA
-    each: more MMAs per stage than a warp has lanes; runs of tile rows across,
-    below and around the middle of the group are one MMA each."""
-    m, k, n = 256, 16 * 37, 100
-    r = np.arange(16)[rows[0]:rows[1]:rows[2]]
-    brow, bcol = (a.reshape(-1).astype(np.int32) for a in np.meshgrid(r, np.arange(37)))
-    c = wl.integer_problem(900, m, k, n, 16, len(brow))
-    vals = torch.from_numpy(c["vals"]).to(torch.bfloat16).cuda()
-    x = torch.zeros((k, 104), dtype=torch.bfloat16, device="cuda")
-    x[:, :n] = torch.from_numpy(c["X"]).to(torch.bfloat16)
-    w = torch.zeros((16, 37, 16, 16), dtype=torch.float64, device="cuda")
-    w[torch.from_numpy(brow).long(), torch.from_numpy(bcol).long()] = vals.double()
-    want = (w.transpose(1, 2).reshape(m, k) @ x[:, :n].double()).to(torch.bfloat16)
-    p = S.Plan(m, k, n, 16, w_dtype=S.BF16, mode=S.DYNAMIC, nnzb_max=len(brow),
-               rows_per_group=16, stage_geometry=geo)
-    cnt = torch.tensor([len(brow)], dtype=torch.int32, device="cuda")
-    y = p.run(x[:, :n], values=vals, pattern=(cnt, torch.from_numpy(brow).cuda(),
-                                              torch.from_numpy(bcol).cuda()))
-    torch.cuda.synchronize()
-    assert p.status() == 0 and torch.equal(y, want)
-    p.close()
