@@ -147,10 +147,12 @@ static bool b1_prefers_tc(int64_t m, int64_t k, int64_t n_max, spmm_dtype w, spm
 // slots (one per SM for two-column-tile launches, two otherwise; dynamic
 // plans always launch one column tile per CTA, so they pass wide = false),
 // measured by waves x rows per unit, ceil(q U / S) / q; 0 keeps the equal
-// partition.  Groups keep at least 12 rows and a new count must be at least
+// partition.  Groups keep at least 10 rows and a new count must be at least
 // 3 % better.  At m = k = 4096, n = 2048 this gives 19 groups of 13-14 rows
 // (19 x 8 units on 152 SMs), 2-8 % faster on every point of the sweep than
-// 16 groups of 16.
+// 16 groups of 16; at b = 4, d = 1/8, n = 1500 25 groups of 10-11 rows take
+// 47.5 us, 21 of 12-13 (one column tile per CTA, as n is no multiple of 64)
+// took 53.2.
 static int64_t auto_groups(int64_t mt, int64_t n_max, int sms, bool wide) {
     if (sms <= 0 || mt <= 0) return 0;
     const int64_t ntn = std::max<int64_t>(1, (n_max + kNTile - 1) / kNTile);
@@ -159,7 +161,7 @@ static int64_t auto_groups(int64_t mt, int64_t n_max, int sms, bool wide) {
     if (q16 * ntn < sms) return 0;   // small problems: the rows-per-group rule
     auto cost = [&](int64_t q) { return (double)((q * U + S - 1) / S) / (double)q; };
     int64_t best = q16;
-    for (int64_t q = q16 + 1; q <= mt / 12; ++q)
+    for (int64_t q = q16 + 1; q <= mt / 10; ++q)
         if (cost(q) < cost(best)) best = q;
     return cost(best) < 0.97 * cost(q16) ? best : 0;
 }
@@ -590,7 +592,7 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
                     const bool can_wide = o.col_tiles == 2
                                               ? n_max > kNTile
                                               : (w_dtype != SPMM_E4M3 && o.col_tiles != 1 &&
-                                                 n_max > kNTile && n_max % 64 == 0);
+                                                 n_max > kNTile);
                     const int64_t qn = auto_groups(mt, n_max, p->sm_count, false);
                     const int64_t qw = can_wide ? auto_groups(mt, n_max, p->sm_count, true) : qn;
                     if (qn == qw) {
@@ -620,6 +622,7 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
                         choose_tc_shape(m, k, b, p->nnzb, pattern->brow, pattern->bcol,
                                         std::max<int64_t>(n_max, 1), p->sm_count, ct, p->R);
                     p->R = sh.rows;
+                    p->groups = sh.groups;
                     splits = sh.splits > 1 ? sh.splits : 0;
                     auto_split = splits > 0;
                     p->auto_wide = o.col_tiles == 0 && sh.col_tiles == 2;

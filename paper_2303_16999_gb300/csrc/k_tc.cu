@@ -136,6 +136,9 @@ namespace {
 #ifndef SPMM_TC_TILES8_S
 #define SPMM_TC_TILES8_S 26 // the most that leaves two CTAs per SM
 #endif
+// Deep launches (one column tile, one CTA per SM): the same stages, as many
+// as an SM's shared memory holds.
+constexpr int kDeepStages = 4, kDeepStages8 = 6, kDeepStages8S = 4;
 constexpr int kSlabBytes = kTile * kNTile * 2;                    // 4096: 16 k x 128 n, 16-bit
 constexpr int kTileBytes8 = kTile * kTile;                        // 256: E4M3 tile, row-major
 constexpr int kScaleBytes = 16 * 4;                               // per slot: 4 x 4 sub-square scales
@@ -149,10 +152,13 @@ constexpr int kMaxBatch = 64;                                     // problems pe
 // loaded, which the converter warps expand into the 16-bit area.
 // GEO: 0 = dense, 1 = sparse; 2 and 3 = the same over two column tiles per
 // CTA ("wide": one CTA per SM, each W tile serves 256 columns of n; the
-// same entry and tile caps, hence the same stage records, as GEO - 2).
+// same entry and tile caps, hence the same stage records, as GEO - 2);
+// 4 and 5 = GEO - 4 with a ring of kDeepStages stages ("deep": one CTA per
+// SM, for launches of at most one work unit per SM).
 template <bool W8, int GEO> struct StageGeom {
     static constexpr int base = GEO & 1;            // dense (0) or sparse (1) tiles
-    static constexpr int sets = GEO >= 2 ? 2 : 1;   // column tiles per CTA
+    static constexpr bool deep = GEO >= 4;
+    static constexpr int sets = GEO >= 2 && !deep ? 2 : 1;   // column tiles per CTA
     // X producer warps per column tile in wide CTAs: sparse-tile stages
     // carry up to 2 x 8 separate slab copies, so two warps share each tile's
     static constexpr int xprod = GEO == 3 ? 2 : 1;
@@ -161,7 +167,8 @@ template <bool W8, int GEO> struct StageGeom {
     static constexpr int mma_warps = 2 * sets;      // one per row half and column tile
     // E4M3 weights: the same stage shapes whether a CTA covers one column
     // tile or two (its W tiles, codes and scales serve both)
-    static constexpr int stages = W8 ? (base ? SPMM_TC_STAGES8_S : SPMM_TC_STAGES8)
+    static constexpr int stages = deep ? (W8 ? (base ? kDeepStages8S : kDeepStages8) : kDeepStages)
+                                     : W8 ? (base ? SPMM_TC_STAGES8_S : SPMM_TC_STAGES8)
                                      : GEO == 3   ? SPMM_TC_STAGES_WS
                                        : GEO == 2 ? SPMM_TC_STAGES_W
                                        : GEO      ? SPMM_TC_STAGES_S
@@ -944,20 +951,32 @@ __global__ void quantize_e4m3_kernel(const U *__restrict__ src, int64_t nnzb, in
 }
 
 // Wide launches (two column tiles per CTA, one CTA per SM, each W tile read
-// once per 256 columns of n): static 16-bit plans over a 3-D X map (n a
-// multiple of 64) with n > 128.  Automatically for dense-tile plans with
+// once per 256 columns of n): static 16-bit plans with n > 128, over either X
+// map (a dense-tile stage has joint boxes in both: 4096 x 4096, b = 4, d = 1/8,
+// n = 2000 55.5 -> 50.3 us).  Automatically for dense-tile plans with
 // enough work units that halving them still fills the SMs (a wide CTA does
 // the work of two narrow ones, which share an SM otherwise).  Measured at
 // m = k = 4096, n = 2048, every dense-tile point of the sweep ran 5-11 %
 // faster wide; every sparse-tile point 6-11 % slower (two 86 KB stages per
 // CTA, against two narrow CTAs whose stages interleave).
-bool use_wide(const spmm_plan *p, int64_t n, int x3d) {
+bool use_wide(const spmm_plan *p, int64_t n) {
     if (p->col_tiles == 1 || p->mode != SPMM_STATIC || n <= kNTile) return false;
     // forced: any n > 128 (2-D X maps included) and E4M3 weights as well
     if (p->col_tiles == 2 || p->auto_wide) return true;
-    if (!x3d || p->wdt == SPMM_E4M3) return false;
+    if (p->wdt == SPMM_E4M3) return false;
     const int64_t units = p->n_items * ((n + kNTile - 1) / kNTile);
     return p->tc_geo == 0 && 2 * units >= (int64_t)SPMM_TC_WIDE_MIN * p->sm_count;
+}
+
+// Deep launches: with at most one work unit per SM no second CTA shares an
+// SM, so the unit's ring takes all of its shared memory (four stages of 16-bit
+// weights instead of two).  152 units of 4096 x 4096, n = 1000, 19 groups of
+// tile rows: b = 4, d = 1/8 44.0 -> 38.8 us, b = 16, d = 1/4 35.5 -> 31.4; 2048 x
+// 2048, b = 4, d = 1/4, n = 2000 24.3 -> 22.8; units of few stages (4096 x
+// 4096, b = 4, d = 1/8, n = 200 in 128 units) take the same time either way.
+// Static plans alone: a dynamic call's item count is known on the device.
+bool use_deep(const spmm_plan *p, int64_t units) {
+    return p->mode == SPMM_STATIC && units <= p->sm_count;
 }
 
 void fill_prob(TcProb &P, const spmm_plan *p, void *Y, int64_t n, int64_t ldy, int x3d,
@@ -1009,6 +1028,13 @@ cudaError_t launch_batch(const TcBatch &B, int sm_count, cudaStream_t s) {
 
 template <typename T>
 cudaError_t launch_geo(const TcBatch &B, int geo, bool w8, int sm_count, cudaStream_t s) {
+    if (geo >= 4) {
+        if (w8)
+            return geo == 5 ? launch_batch<T, true, 5>(B, sm_count, s)
+                            : launch_batch<T, true, 4>(B, sm_count, s);
+        return geo == 5 ? launch_batch<T, false, 5>(B, sm_count, s)
+                        : launch_batch<T, false, 4>(B, sm_count, s);
+    }
     if (w8) {
         if (geo == 3) return launch_batch<T, true, 3>(B, sm_count, s);
         if (geo == 2) return launch_batch<T, true, 2>(B, sm_count, s);
@@ -1046,7 +1072,7 @@ cudaError_t launch_tc(const spmm_plan *p, const void *X, int64_t n, int64_t ldx,
     int x3d = 0;
     cudaError_t e = encode_x(&B.maps[0], &x3d, p->xdt == SPMM_BF16, X, p->k, n, ldx);
     if (e != cudaSuccess) return e;
-    const bool wide = use_wide(p, n, x3d);
+    const bool wide = use_wide(p, n);
     e = encode_x(&B.maps4[0], &x3d, p->xdt == SPMM_BF16, X, p->k, n, ldx, kJointSlabs);
     if (e != cudaSuccess) return e;
     fill_prob(B.prob[0], p, Y, n, ldy, x3d);
@@ -1066,7 +1092,8 @@ cudaError_t launch_tc(const spmm_plan *p, const void *X, int64_t n, int64_t ldx,
         e = launch_stage_build(p, s);
         if (e != cudaSuccess) return e;
     }
-    return dispatch_batch(B, p->tc_geo + (wide ? 2 : 0), p->xdt == SPMM_BF16,
+    const bool deep = !wide && use_deep(p, B.total_units);
+    return dispatch_batch(B, p->tc_geo + (wide ? 2 : deep ? 4 : 0), p->xdt == SPMM_BF16,
                           p->wdt == SPMM_E4M3, p->sm_count, s);
 }
 

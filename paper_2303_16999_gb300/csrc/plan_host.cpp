@@ -345,9 +345,10 @@ namespace {
 struct ShapeCost {
     int64_t mt, kt, n;
     double sms;
-    // E entries and S tile slots in all groups of R tile rows
-    double us(int64_t R, double E, double S, int ct, int64_t splits) const {
-        const int64_t G = (mt + R - 1) / R, ntn = (n + kNTile - 1) / kNTile;
+    // E entries and S tile slots in all G groups; deep: at most one unit per
+    // SM, in the ring of four stages
+    double us(int64_t G, double E, double S, int ct, int64_t splits, bool deep = false) const {
+        const int64_t ntn = (n + kNTile - 1) / kNTile;
         const int64_t nt = (n + kNTile * ct - 1) / (kNTile * ct);
         const double items = (double)(G * splits), slots = ct == 2 ? sms : 2 * sms;
         const double units = items * (double)nt, waves = std::ceil(units / slots);
@@ -358,7 +359,8 @@ struct ShapeCost {
         if (E > 0.9 * (double)(G * kt)) boxes /= 4;   // mostly joint boxes
         const double unit =
             waves * (1.14 + (0.0805 * E + 0.0045 * S) / items * (ct == 2 ? 1.32 : 1));
-        double t = 5.06 + std::max({bytes / 15.2e6 * imb, unit, 0.029 * boxes / sms * imb});
+        double t = 5.06 + std::max({bytes / 15.2e6 * imb, unit * (deep ? 0.87 : 1.0),
+                                    0.029 * boxes / sms * imb});
         if (splits > 1) t += 2.07 + (double)splits * (double)(mt * kTile) * (double)n * 8 / 5.96e6;
         if (ct == 2) t *= 0.95;   // (the model is this much too hard on wide launches)
         return t;
@@ -369,7 +371,7 @@ struct ShapeCost {
 TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
                         const int32_t *bcol, int64_t n, int sms, int ct_only, int default_rows) {
     const int64_t mt = m / kTile, kt = k / kTile;
-    TcShape best{default_rows, 1, ct_only ? ct_only : 1};
+    TcShape best{default_rows, 1, ct_only ? ct_only : 1, 0};
     if (nnzb == 0) return best;
     // tile occupancy of a sample of 16-row bands: one row mask per column
     const int64_t bands = (mt + kMaxGroupRows - 1) / kMaxGroupRows;
@@ -386,15 +388,13 @@ TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t
     std::vector<int> rows;
     std::vector<std::pair<int, int>> ivs;
     double ref = 0, least = 0;
-    const int order[5] = {default_rows, 1, 2, 4, 8};
-    for (int i = 0; i < 6; ++i) {
-        const int R = i < 5 ? order[i] : kMaxGroupRows;
-        if (i > 0 && R == default_rows) continue;
-        // entries of R-row groups, and tile slots from every q-th of them
+    // entries of R-row groups, and tile slots from every q-th of them (of R
+    // that does not divide 16: from the bands' whole groups)
+    auto sample = [&](int R, double &e, double &s) {
         int64_t E = 0, sampled = 0, slots = 0;
         const int64_t every = std::max<int64_t>(1, (int64_t)mask.size() / 512);
         for (size_t c = 0; c < mask.size(); ++c)
-            for (int r0 = 0; r0 < kMaxGroupRows; r0 += R) {
+            for (int r0 = 0; r0 + R <= kMaxGroupRows; r0 += R) {
                 const uint32_t g = (mask[c] >> r0) & ((1u << R) - 1);
                 if (!g) continue;
                 if (E++ % every) continue;
@@ -405,7 +405,15 @@ TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t
                 ++sampled;
                 for (const auto &iv : ivs) slots += iv.second;
             }
-        const double e = (double)E * scale, s = sampled ? e * (double)slots / (double)sampled : 0;
+        e = (double)E * scale * kMaxGroupRows / (double)(kMaxGroupRows / R * R);
+        s = sampled ? e * (double)slots / (double)sampled : 0;
+    };
+    const int order[5] = {default_rows, 1, 2, 4, 8};
+    for (int i = 0; i < 6; ++i) {
+        const int R = i < 5 ? order[i] : kMaxGroupRows;
+        if (i > 0 && R == default_rows) continue;
+        double e = 0, s = 0;
+        sample(R, e, s);
         const int64_t G = (mt + R - 1) / R;
         for (int ct = 1; ct <= 2; ++ct) {
             if ((ct_only && ct != ct_only) || (ct == 2 && (n <= kNTile || (!ct_only && n > 512))))
@@ -414,14 +422,37 @@ TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t
             const int64_t kmax = std::max<int64_t>(1, (ct == 2 ? sms : 2 * sms) / (G * nt));
             for (int64_t q : {(int64_t)1, kmax / 3, kmax / 2, kmax * 2 / 3, kmax}) {
                 if (q < 1 || q > 1024 || q > std::max<int64_t>(1, kt / 4)) continue;
-                const double t = cost.us(R, e, s, ct, q);
+                const double t = cost.us(G, e, s, ct, q);
                 if (ref == 0) ref = least = t;   // the default: first of all
                 // something else only for a clear gain over the default
                 if (t < least && t < 0.9 * ref) {
                     least = t;
-                    best = TcShape{R, (int)q, ct};
+                    best = TcShape{R, (int)q, ct, 0};
                 }
             }
+        }
+    }
+    // near-equal groups that make one unit for every SM (each then has all of
+    // its shared memory: a deep launch) or for every CTA slot, unsplit.  The
+    // first has to promise 3 % only: one full wave is the model's best ground
+    // (it takes 0.87 of the two-stage ring's time for a unit's stages).
+    // 4096 x 4096, n = 1000: b = 4, d = 1/8 46.9 -> 38.8 us, b = 8 43.2 -> 37.6,
+    // b = 16, d = 1/4 36.3 -> 31.4, b = 8, d = 1/16 35.5 -> 30.0.
+    const int64_t ntn = (n + kNTile - 1) / kNTile;
+    for (int per = 1; per <= 2; ++per) {
+        const int64_t G = std::min<int64_t>(per * (int64_t)sms / ntn, mt);
+        if (ct_only == 2 || G <= 0 || (mt + G - 1) / G > kMaxGroupRows) continue;
+        const bool deep = G * ntn <= sms;
+        if (deep && kt < 64) continue;   // (too few stages to gain from the ring)
+        const int64_t R = (mt + G - 1) / G;
+        double e = 0, s = 0;
+        sample((int)R, e, s);
+        // (sampled at the larger groups' rows: mt / R of them, not G)
+        const double f = (double)mt / (double)(G * R);
+        const double t = cost.us(G, e / f, s, 1, 1, deep);
+        if (t < least && t < (deep ? 0.97 : 0.9) * ref) {
+            least = t;
+            best = TcShape{(int)R, 1, 1, G};
         }
     }
     return best;

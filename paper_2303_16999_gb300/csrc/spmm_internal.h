@@ -80,9 +80,11 @@ int64_t count_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *
                       const int32_t *bcol, int64_t R, int64_t groups);
 // launch shape of a static tensor-core plan that 16-row groups alone would
 // not occupy the GPU with: tile rows per group, work items per group along k
-// and column tiles per CTA (ct_only: 0, or the only count allowed)
+// and column tiles per CTA (ct_only: 0, or the only count allowed); groups > 0:
+// that many near-equal groups of at most `rows` rows instead
 struct TcShape {
     int rows, splits, col_tiles;
+    int64_t groups;
 };
 TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
                         const int32_t *bcol, int64_t n, int sms, int ct_only, int default_rows);

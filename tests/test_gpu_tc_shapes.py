@@ -94,3 +94,24 @@ def test_batch_of_split_plans_one_reduction():
     for p, y, want in zip(plans, ys, wants):
         assert p.status() == 0 and torch.equal(y, want)
         p.close()
+
+
+@pytest.mark.parametrize("dt", ["f16", "bf16", "e4m3"])
+@pytest.mark.parametrize("geo", [1, 2])
+@pytest.mark.parametrize("extra", [-1, 0, 1])
+def test_deep_ring_units(dt, geo, extra):
+    """One work unit per SM or fewer takes the deep ring, one more unit does
+    not; 40 entries per unit, so every ring wraps."""
+    g = torch.cuda.get_device_properties(0).multi_processor_count + extra
+    xdt = torch.float16 if dt == "f16" else torch.bfloat16
+    c, vals, x, want = _problem(40 + g, 16 * g, 640, 72, 8, g * 2 * 80 // 2, xdt)
+    if dt != "e4m3":
+        _run(c, vals, x, want, rows_per_group=1, stage_geometry=geo)
+        return
+    p = S.Plan(16 * g, 640, 72, 8, w_dtype=S.E4M3, x_dtype=S.BF16, brow=c["brow"], bcol=c["bcol"],
+               kernel="tc", rows_per_group=1, stage_geometry=geo)
+    p.pack(vals.to(torch.float8_e4m3fn), torch.ones(len(c["brow"]), device="cuda"))
+    y = p.run(x)
+    torch.cuda.synchronize()
+    assert p.status() == 0 and torch.equal(y, want)
+    p.close()
