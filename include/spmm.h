@@ -122,8 +122,8 @@ typedef struct {
     int32_t col_tiles;            /* TC, static plans: 128-column tiles of n per CTA.  1 = one;
                                      2 = two whenever n > 128 (16-bit or E4M3 weights): the two
                                      tiles share every W stage (and its E4M3 expansion), one CTA
-                                     per SM; 0 = automatic (two for 16-bit dense-tile plans with n
-                                     a multiple of 64 and enough work units).  Results are
+                                     per SM; 0 = automatic (two for 16-bit dense-tile plans with
+                                     n > 128 and enough work units).  Results are
                                      identical either way.  Other values SPMM_ERR_ARG. */
     int64_t groups;               /* TC plans: split the m/16 tile rows into exactly this many
                                      groups of near-equal size (sizes differ by at most one, larger

@@ -337,7 +337,9 @@ int64_t count_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *
 //                              unit, 1.32 times that over two column tiles),
 //                     0.029 per TMA box of an SM x imbalance)       [us]
 //          + for split groups 2.07 + partials written and read at 5.96 TB/s.
-// Another shape than the rows-per-group rule's has to promise 10 % less.  On
+// Another shape than the rows-per-group rule's has to promise 20 % less, and
+// groups are split only where that rule shrinks them below 4 rows (6064 x 6800,
+// b = 8, d = 1/4, n = 319, 4 rows: 53.6 us, split 76.2).  On
 // those products the pick takes 1.02 times the best shape's time on average
 // and 0.80 times the rule's: 4096 x 16384, b = 8, d = 1/8: n = 24 62.0 -> 23.4
 // us, n = 200 82.3 -> 39.7; 4096 x 4096, b = 4, d = 1/8, n = 100 48.1 -> 16.4.
@@ -414,7 +416,9 @@ TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t
         if (i > 0 && R == default_rows) continue;
         double e = 0, s = 0;
         sample(R, e, s);
-        const int64_t G = (mt + R - 1) / R;
+        // (the equal partition makes up to a few groups more than mt / R: 27 of
+        // 379 tile rows at R = 16, and units beyond a wave cost another)
+        const int64_t G = (int64_t)group_partition(mt, R).size();
         for (int ct = 1; ct <= 2; ++ct) {
             if ((ct_only && ct != ct_only) || (ct == 2 && (n <= kNTile || (!ct_only && n > 512))))
                 continue;
@@ -422,10 +426,11 @@ TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t
             const int64_t kmax = std::max<int64_t>(1, (ct == 2 ? sms : 2 * sms) / (G * nt));
             for (int64_t q : {(int64_t)1, kmax / 3, kmax / 2, kmax * 2 / 3, kmax}) {
                 if (q < 1 || q > 1024 || q > std::max<int64_t>(1, kt / 4)) continue;
+                if (q > 1 && default_rows >= 4) continue;   // (re-reads of X are few there)
                 const double t = cost.us(G, e, s, ct, q);
                 if (ref == 0) ref = least = t;   // the default: first of all
                 // something else only for a clear gain over the default
-                if (t < least && t < 0.9 * ref) {
+                if (t < least && t < 0.8 * ref) {
                     least = t;
                     best = TcShape{R, (int)q, ct, 0};
                 }
@@ -438,13 +443,18 @@ TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t
     // (it takes 0.87 of the two-stage ring's time for a unit's stages).
     // 4096 x 4096, n = 1000: b = 4, d = 1/8 46.9 -> 38.8 us, b = 8 43.2 -> 37.6,
     // b = 16, d = 1/4 36.3 -> 31.4, b = 8, d = 1/16 35.5 -> 30.0.
+    // 16-bit weights alone (ct_only: E4M3): one CTA per SM halves the warps that
+    // expand E4M3 tiles (2256 x 6208, b = 8, d = 1/8, n = 1695: 106 us deep, 84 not).
     const int64_t ntn = (n + kNTile - 1) / kNTile;
     for (int per = 1; per <= 2; ++per) {
         const int64_t G = std::min<int64_t>(per * (int64_t)sms / ntn, mt);
-        if (ct_only == 2 || G <= 0 || (mt + G - 1) / G > kMaxGroupRows) continue;
+        if (ct_only || G <= 0 || (mt + G - 1) / G > kMaxGroupRows) continue;
         const bool deep = G * ntn <= sms;
-        if (deep && kt < 64) continue;   // (too few stages to gain from the ring)
         const int64_t R = (mt + G - 1) / G;
+        // (few stages do not gain from the ring; in groups of few rows two CTAs
+        // per SM issue more: 4096 x 4096, b = 4, d = 1/8, n = 640 34.6 us in 30
+        // groups, 29.6 in 60)
+        if (deep && (kt < 64 || R < 12)) continue;
         double e = 0, s = 0;
         sample((int)R, e, s);
         // (sampled at the larger groups' rows: mt / R of them, not G)
