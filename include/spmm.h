@@ -324,7 +324,8 @@ int64_t spmm_bucket_size(int64_t m, int64_t k, int64_t d_max_num, int64_t d_max_
  * stage records cut for it (built once per plan on first use; results are
  * identical).  The tensor-core launch's CTAs walk one schedule of
  * (problem, work item, n tile) units, precomputed on the host when the
- * plan set is first run (costliest units first) and cached; each CTA takes
+ * plan set is first run (costliest units first) and cached until one of
+ * its plans is destroyed; each CTA takes
  * every gridDim-th unit of it (no atomic work queue).  Each problem with
  * rows split over several work items adds one reduction launch.  d_X[i],
  * n[i], ldx[i], d_Y[i], ldy[i] as in spmm_run (ldx/ldy may be NULL for

@@ -762,6 +762,7 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
 
 void spmm_plan_destroy(spmm_plan *plan) {
     if (plan && plan->ran && plan->done) cudaEventSynchronize(plan->done);
+    if (plan && plan->kernel == SPMM_KERNEL_TC) forget_schedules(plan);
     free_plan(plan);
 }
 

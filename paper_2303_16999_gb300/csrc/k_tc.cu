@@ -1052,7 +1052,10 @@ cudaError_t dispatch_batch(const TcBatch &B, int geo, bool bf16, bool w8, int sm
 
 // Cached launch schedules of batches: (problem, unit) pairs of all problems,
 // costliest first (item cost = tile slots + entries, as the planner defines
-// it), then by problem and unit.  Keyed by the plans and each problem's n.
+// it), then by problem and unit.  Keyed by the plans and each problem's n; a
+// schedule lives as long as every plan it names (forget_schedules): another
+// plan at a freed address may have another number of work items, and a launch
+// would read past the array.
 struct SchedKey {
     std::vector<const void *> plans;
     std::vector<int64_t> n;
@@ -1061,9 +1064,24 @@ struct SchedKey {
     }
 };
 std::mutex g_sched_mu;
-std::map<SchedKey, int32_t *> g_sched;
+// (never destructed: plans may be destroyed while the process exits)
+std::map<SchedKey, int32_t *> &g_sched = *new std::map<SchedKey, int32_t *>;
 
 }  // namespace
+
+// Called before plan p is freed, when its last launch has completed.
+void forget_schedules(const spmm_plan *p) {
+    std::lock_guard<std::mutex> lk(g_sched_mu);
+    for (auto it = g_sched.begin(); it != g_sched.end();) {
+        const std::vector<const void *> &v = it->first.plans;
+        if (std::find(v.begin(), v.end(), p) == v.end()) {
+            ++it;
+            continue;
+        }
+        if (it->second) cudaFree(it->second);
+        it = g_sched.erase(it);
+    }
+}
 
 cudaError_t launch_tc(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, void *Y,
                       int64_t ldy, cudaStream_t s) {
