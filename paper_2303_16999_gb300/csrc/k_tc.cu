@@ -1119,7 +1119,7 @@ namespace {
 cudaError_t launch_tc_group(int count, spmm_plan *const *plans, const void *const *X,
                             const int64_t *n, const int64_t *ldx, void *const *Y,
                             const int64_t *ldy, cudaStream_t s, bool schedule, int geo);
-cudaError_t ensure_alt_records(spmm_plan *p, int geo, cudaStream_t s);
+cudaError_t ensure_alt_records(spmm_plan *p, int geo);
 }
 
 // Plans of both stage geometries in one launch, in the geometry that holds
@@ -1155,7 +1155,7 @@ cudaError_t launch_tc_batch(int count, spmm_plan *const *plans, const void *cons
         const int geo = units[1] > units[0] ? 1 : 0;
         for (int i = 0; i < c; ++i) {
             if (gp[i]->tc_geo == geo) continue;
-            cudaError_t e = ensure_alt_records(gp[i], geo, s);
+            cudaError_t e = ensure_alt_records(gp[i], geo);
             if (e != cudaSuccess) return e;
         }
         cudaError_t e = launch_tc_group(c, gp, gx, gn, glx, gy, gly, s, schedule, geo + 2 * wide);
@@ -1166,9 +1166,13 @@ cudaError_t launch_tc_batch(int count, spmm_plan *const *plans, const void *cons
 
 namespace {
 // Stage records of plan p cut for stage geometry `geo` (not its own) into
-// d_srec_alt / d_sprog_alt, allocated on first use (outside any stream
-// capture: the first batched launch of a plan set allocates).
-cudaError_t ensure_alt_records(spmm_plan *p, int geo, cudaStream_t s) {
+// d_srec_alt / d_sprog_alt, built on first use (outside any stream capture:
+// the first batched launch of a plan set allocates).  They are complete when
+// this returns: a server launches one plan on several streams at a time, and
+// nothing orders a second stream behind the one that would have built them.
+std::mutex g_alt_mu;
+cudaError_t ensure_alt_records(spmm_plan *p, int geo) {
+    std::lock_guard<std::mutex> lk(g_alt_mu);
     if (p->alt_geo == geo) return cudaSuccess;
     const int64_t E = std::max<int64_t>(p->n_entries, 1);
     if (!p->d_srec_alt) {
@@ -1190,13 +1194,19 @@ cudaError_t ensure_alt_records(spmm_plan *p, int geo, cudaStream_t s) {
                              : (geo ? StageGeom<false, 1>::tiles : StageGeom<false, 0>::tiles);
     const int ent_cap = w8 ? (geo ? StageGeom<true, 1>::ent : StageGeom<true, 0>::ent)
                            : (geo ? StageGeom<false, 1>::ent : StageGeom<false, 0>::ent);
-    if (p->n_items > 0)
-        pdl_launch(stage_build_kernel, dim3((unsigned)p->n_items), dim3(kBuildWarps * 32), 0, s,
+    if (p->n_items > 0) {
+        cudaStream_t s = nullptr;
+        cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return e;
+        e = pdl_launch(stage_build_kernel, dim3((unsigned)p->n_items), dim3(kBuildWarps * 32), 0, s,
             p->d_items, p->n_items, (const int32_t *)nullptr, p->d_status, p->d_ent_col,
             p->d_ent_tbeg, p->d_ent_cover, ent_cap, tiles_cap, p->d_srec_alt, p->d_sprog_alt);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) p->alt_geo = geo;
-    return e;
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        cudaStreamDestroy(s);
+        if (e != cudaSuccess) return e;
+    }
+    p->alt_geo = geo;
+    return cudaSuccess;
 }
 
 cudaError_t launch_tc_group(int count, spmm_plan *const *plans, const void *const *X,
