@@ -112,7 +112,9 @@ typedef struct {
     int32_t rows_per_group;       /* TC: tile rows (16 rows each) per group, 1..16; 0 = planner's choice
                                      (static plans whose 16-row groups would not occupy the GPU: rows
                                      per group and splits along k together) */
-    int32_t max_per_item;         /* TC: entries per work item; GATHER: blocks per row item; 0 = planner's choice */
+    int32_t max_per_item;         /* TC: entries per work item; GATHER: blocks per row item; 0 = planner's
+                                     choice (GATHER: of the kernel as well, see gather_form in the
+                                     plan's info; a given length runs the items) */
     int32_t host_only;            /* 1 = build the static plan on the host only (no device memory, no
                                      CUDA calls): for inspection with spmm_plan_get_array */
     int32_t transposed;           /* 1 = the plan applies W^T: spmm_run computes Z = W^T.Y (Z k x n,
@@ -269,6 +271,12 @@ typedef struct {
                                      GATHER plans with k <= 65536 (a 16-bit copy of col_idx,
                                      read by the kernels that keep X in shared memory),
                                      else 4 */
+    int32_t auto_col_tiles;       /* TC, col_tiles 0: 2 when the planner chose two column tiles
+                                     per CTA (for n > 128) with the plan's groups and splits,
+                                     else 0 (large plans: by the launch, see col_tiles) */
+    int32_t gather_form;          /* GATHER: a call with n = n_max, 16-byte aligned X and rows of
+                                     X padded to 8 values 1 = keeps X in shared memory, one pass
+                                     over equal row ranges, 0 = runs the row items */
 } spmm_plan_info;
 
 spmm_status spmm_plan_get_info(const spmm_plan *plan, spmm_plan_info *info);

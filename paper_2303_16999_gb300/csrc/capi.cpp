@@ -179,6 +179,54 @@ static bool col16_plan(const spmm_plan *p) {
     return p->kernel == SPMM_KERNEL_GATHER && p->mode == SPMM_STATIC && p->k / p->b <= 65536;
 }
 
+// Where each of the kGxParts parts of k starts in every row.
+static std::vector<int32_t> gx_pointers(const spmm_plan *p) {
+    const HostPlan &hp = p->hp;
+    const int64_t pw = (p->k + kGxParts - 1) / kGxParts, m = p->m;
+    std::vector<int32_t> ptr(m * kGxParts + 1);
+    for (int64_t r = 0; r < m; ++r) {
+        int32_t i = hp.row_ptr[r];
+        for (int q = 0; q < kGxParts; ++q) {
+            ptr[r * kGxParts + q] = i;
+            i = (int32_t)(std::lower_bound(hp.col_idx.begin() + i,
+                                           hp.col_idx.begin() + hp.row_ptr[r + 1],
+                                           (q + 1) * pw) - hp.col_idx.begin());
+        }
+    }
+    ptr[m * kGxParts] = hp.row_ptr[m];
+    return ptr;
+}
+
+// How a plan's non-zeros lie over row ranges, slices of k and rows (GxLoad).
+static GxLoad gx_load(const spmm_plan *p) {
+    const HostPlan &hp = p->hp;
+    const int64_t m = p->m;
+    const std::vector<int32_t> ptr = gx_pointers(p);
+    GxLoad g;
+    g.on = true;
+    for (int64_t r = 0; r < m; ++r)
+        g.longest_row = std::max<int64_t>(g.longest_row, hp.row_ptr[r + 1] - hp.row_ptr[r]);
+    std::vector<int64_t> upto(m + 1);
+    for (int c = 0; c < 3; ++c) {
+        const int cs = 1 << c, per = kGxParts / cs;
+        for (int q = 0; q < cs; ++q) {
+            upto[0] = 0;
+            for (int64_t r = 0; r < m; ++r) {
+                const int64_t nz = ptr[r * kGxParts + (q + 1) * per] - ptr[r * kGxParts + q * per];
+                g.row_slice[c] = std::max(g.row_slice[c], nz);
+                upto[r + 1] = upto[r] + nz;
+            }
+            for (int j = 0; j < 8; ++j) {
+                const int64_t rr = (m + (1 << j) - 1) / (1 << j);
+                for (int64_t r = 0; r < m; r += rr)
+                    g.heavy[c][j] =
+                        std::max(g.heavy[c][j], upto[std::min(m, r + rr)] - upto[r]);
+            }
+        }
+    }
+    return g;
+}
+
 static spmm_status upload_plan(spmm_plan *p) {
     HostPlan &hp = p->hp;
     cudaError_t e = cudaSuccess;
@@ -194,20 +242,7 @@ static spmm_status upload_plan(spmm_plan *p) {
         // the b = 1 gather's column indices in half the bytes
         const std::vector<uint16_t> c16(hp.col_idx.begin(), hp.col_idx.end());
         e = upload(p, &p->d_col16, c16);
-        // where each part of k starts in every row
-        const int64_t pw = (p->k + kGxParts - 1) / kGxParts, m = p->m;
-        std::vector<int32_t> ptr(m * kGxParts + 1);
-        for (int64_t r = 0; r < m; ++r) {
-            int32_t i = hp.row_ptr[r];
-            for (int q = 0; q < kGxParts; ++q) {
-                ptr[r * kGxParts + q] = i;
-                i = (int32_t)(std::lower_bound(hp.col_idx.begin() + i,
-                                               hp.col_idx.begin() + hp.row_ptr[r + 1],
-                                               (q + 1) * pw) - hp.col_idx.begin());
-            }
-        }
-        ptr[m * kGxParts] = m ? hp.row_ptr[m] : 0;
-        if (e == cudaSuccess) e = upload(p, &p->d_gx_ptr, ptr);
+        if (e == cudaSuccess && p->gx.on) e = upload(p, &p->d_gx_ptr, gx_pointers(p));
     }
     if (p->kernel == SPMM_KERNEL_TC) {
         UP(d_grp_row0, grp_row0);
@@ -583,6 +618,8 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
                 const int64_t avg = mb ? (p->nnzb + mb - 1) / mb : 0;
                 p->C = o.max_per_item ? o.max_per_item : (int)std::max<int64_t>(64, 2 * avg);
                 build_row_plan(mb, p->C, true, p->hp);
+                // (items of a given length: the kernels that run them)
+                if (col16_plan(p) && !o.max_per_item) p->gx = gx_load(p);
             } else if (kernel == SPMM_KERNEL_TC) {
                 p->groups = o.groups;
                 if (!p->groups && !o.rows_per_group && p->sm_count > 0) {
@@ -858,7 +895,7 @@ static spmm_status launch_product(spmm_plan *p, const void *d_X, int64_t n, int6
                               : launch_plain(p, d_X, n, ldx, d_Y, ldy, s);
             break;
         case SPMM_KERNEL_GATHER:
-            whole = gather_xs_takes(p, n);
+            whole = gather_xs_takes(p, d_X, n, ldx, d_Y, ldy);
             e = whole ? launch_gather_xs(p, d_X, n, ldx, d_Y, ldy, s)
                       : launch_gather(p, d_X, n, ldx, d_Y, ldy, s);
             break;
@@ -1091,6 +1128,9 @@ spmm_status spmm_plan_get_info(const spmm_plan *cp, spmm_plan_info *info) {
     i.sddmm_form = sddmm_gathers(p) ? 1 : 0;
     i.row_begin = p->row_end ? p->row_begin : 0;
     i.row_end = p->row_end ? p->row_end : p->m;
+    i.auto_col_tiles = p->auto_wide ? 2 : 0;
+    i.gather_form =
+        gather_xs_takes(p, nullptr, p->n_max, (p->n_max + 7) / 8 * 8, nullptr, p->n_max) ? 1 : 0;
     *info = i;
     return SPMM_OK;
 }

@@ -701,16 +701,11 @@ cudaError_t gather_launch(const spmm_plan *p, const void *X, int64_t n, int64_t 
 template <typename T>
 cudaError_t gather_dispatch(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, void *Y,
                             int64_t ldy, cudaStream_t s) {
-    // widest vector that keeps every lane's load aligned and inside its row
     constexpr int Vmax = 16 / sizeof(T);
-    auto ok = [&](int V) {
-        const int64_t bytes = V * (int64_t)sizeof(T);
-        return n % V == 0 && ldx % V == 0 && ldy % V == 0 &&
-               ((uintptr_t)X % bytes) == 0 && ((uintptr_t)Y % bytes) == 0;
-    };
-    if (Vmax >= 8 && ok(8)) return gather_launch<T, (Vmax >= 8 ? 8 : 1)>(p, X, n, ldx, Y, ldy, s);
-    if (ok(4)) return gather_launch<T, 4>(p, X, n, ldx, Y, ldy, s);
-    if (ok(2)) return gather_launch<T, 2>(p, X, n, ldx, Y, ldy, s);
+    const int V = gather_vector(p, X, n, ldx, Y, ldy);
+    if (Vmax >= 8 && V == 8) return gather_launch<T, (Vmax >= 8 ? 8 : 1)>(p, X, n, ldx, Y, ldy, s);
+    if (V == 4) return gather_launch<T, 4>(p, X, n, ldx, Y, ldy, s);
+    if (V == 2) return gather_launch<T, 2>(p, X, n, ldx, Y, ldy, s);
     return gather_launch<T, 1>(p, X, n, ldx, Y, ldy, s);
 }
 
@@ -809,6 +804,17 @@ cudaError_t launch_plain(const spmm_plan *p, const void *X, int64_t n, int64_t l
     pdl_launch(plain_f32_kernel, dim3(grid), dim3(128), 0, s, p->d_row_ptr, p->d_col_idx,
         (const float *)p->d_packed, (const float *)X, ldx, (float *)Y, ldy, p->m, n, p->b);
     return cudaGetLastError();
+}
+
+// The widest vector that keeps every lane's load aligned and inside its row.
+int gather_vector(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, const void *Y,
+                  int64_t ldy) {
+    const int es = (int)dtype_size(p->xdt);
+    for (int V = 16 / es; V > 1; V /= 2)
+        if (n % V == 0 && ldx % V == 0 && ldy % V == 0 && (uintptr_t)X % (V * es) == 0 &&
+            (uintptr_t)Y % (V * es) == 0)
+            return V;
+    return 1;
 }
 
 bool gather_ring_fits(const spmm_plan *p, int64_t n) {

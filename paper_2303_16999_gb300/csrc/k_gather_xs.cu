@@ -1,5 +1,5 @@
-// b = 1 gather with X in shared memory (static GATHER plans, more than one
-// 16-byte vector of X per row).
+// b = 1 gather with X in shared memory (static GATHER plans, where the estimate in
+// gather_xs_takes is clearly below the row items' kernels).
 //
 // The gather kernel (k_cudacore.cu) fetches a row of X from L2 for every
 // non-zero: at n = 32 that is 64 bytes per 4-byte non-zero, and L2's latency
@@ -380,26 +380,84 @@ cudaError_t gx_dispatch(const spmm_plan *p, const void *X, int64_t n, int64_t ld
 
 }  // namespace
 
-// Measured at d = 1/16 (1/8 at 4096), FP16, us, gather kernels -> this one: 8192
-// x 8192, n = 12: 29.5 -> 17.0, n = 32: 43.2 -> 25.0, n = 100: 181 -> 87; 4096
-// x 4096, n = 9: 38.8 -> 10.4, n = 64: 66.2 -> 20.0; 16384 x 16384, n = 32: 146
-// -> 104; 1024 x 1024, n = 32: 7.0 -> 4.9; 512 x 512, n = 9: 4.0 -> 4.3, n = 64:
-// 5.2 -> 4.5.  One vector of X per row (n = 1, 2, 4, 8) stays with the ring
-// kernel where X fits that one's memory (8192 x 8192, n = 1: 8.3 against 13.5;
-// 16384 x 16384, n = 8, where it does not: 50.2 -> 36.0).  FP32 takes it while
-// a slice holds as many columns as one warp covers (4096 x 4096, n = 64: 58.6
-// -> 32.4; 8192 x 8192, n = 12: 29.0 -> 24.7, but n = 32, in two chunks: 40.7
-// against 43.6) and more than one vector per row.
-bool gather_xs_takes(const spmm_plan *p, int64_t n) {
-    if (!p->d_gx_ptr || n < 1) return false;
+// Whether this kernel takes a call, or the row items' kernels (k_cudacore.cu)
+// keep it.  Either can be several times as fast: this one copies all of X's
+// slice into every CTA and walks equal ranges of rows, so few non-zeros per row,
+// or a pattern that loads one range, one slice or one row, leave it waiting;
+// the item kernels fetch a row of X per non-zero, from items cut to length.  So
+// both times are estimated, and this kernel has to promise 15 % less.  The
+// terms were fitted to products timed with both kernels on a GB300 (m 100 to
+// 16384, k 100 to 53000, n 1 to 300, d 1/4 to 1/4096; uniform, banded, diagonal
+// and skewed patterns).  On 1411 of them the estimates' rms errors are 10 to 21
+// %, the pick takes 1.04 times the faster kernel's time on average, and it is
+// more than 3 % slower than the items once (0.92 of their speed).  us, items -> this:
+// d = 1/16, FP16, 8192 x 8192: n = 12 29.5 -> 17.0, n = 32 43.2 -> 25.0, n = 100 181
+// -> 87; 4096 x 4096, d = 1/8, n = 64: 66.2 -> 20.0, FP32 58.6 -> 32.4.  Kept by
+// the items: 8192 x 8192, d = 1/1024, n = 100: 7.4 (48.0 here); 4096 x 4096, d =
+// 1/256, FP32, n = 64: 5.8 (15.4); 2048 x 2048, d = 1/64, n = 20: 3.9 (8.0); 4096 x
+// 4096, d = 1/16 near the diagonal, FP32, n = 64: 27.9 (53.4).
+static double gx_us(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, int ln, int cs) {
+    const bool f32 = p->xdt == SPMM_F32;
+    const int es = f32 ? 4 : 2, V = 16 / es, c = cs >> 1;   // c = log2 cs
+    const int64_t cl = cs == 1 ? gx_clusters<1>() : cs == 2 ? gx_clusters<2>() : gx_clusters<4>();
+    const int64_t nch = (n + ln * V - 1) / (ln * V), ranges = std::max<int64_t>(1, cl / nch);
+    const int64_t rr = (p->m + ranges - 1) / ranges;
+    const double waves = (double)(((p->m + rr - 1) / rr * nch + cl - 1) / cl);
+    int j = 0;
+    while (j < 7 && (2 << j) <= ranges) ++j;
+    const double heavy = std::max((double)p->gx.heavy[c][j] * (double)(1 << j) / (double)ranges,
+                                  (1 << j) < ranges ? (double)p->gx.heavy[c][std::min(j + 1, 7)] : 0);
+    // X: 16-byte pieces (rows of an odd number of them are slow to copy), or
+    // values one by one
+    const double pieces = (double)p->k / cs * ln;
+    const int64_t row = ldx * es;
+    const double copy = (uintptr_t)X % 16 || row % 16 ? 1.45e-4 * V
+                        : row % 32 && ln > 1          ? 6.7e-4
+                                                      : f32 ? 1.75e-4 : 1.9e-4;
+    const double rows = (double)rr, slice = (double)p->gx.row_slice[c];
+    return (f32 ? 3.13 : 2.95) +
+           waves * (pieces * copy + rows / 16 * (f32 ? 0.555 : 0.57) +
+                    rows * ln * (f32 ? 4.5e-4 : 1.8e-3) +
+                    heavy * (f32 ? 6.6e-5 * ln + 1.1e-4 : 3.95e-5 * ln + 1.5e-4) +
+                    slice * (f32 ? 2.5e-4 * ln + 1e-3 : 5e-4 * ln + 1.2e-3));
+}
+
+static double items_us(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, const void *Y,
+                       int64_t ldy) {
+    const bool f32 = p->xdt == SPMM_F32;
+    const double nnz = (double)p->nnzb, reds = (double)p->n_red;
+    const double item = (double)std::min<int64_t>(p->gx.longest_row, p->C);
+    const int64_t vecs = n / gather_vector(p, X, n, ldx, Y, ldy);
+    if (vecs == 1)   // gather1g_kernel (16-bit values)
+        return 3.5 + nnz * (1.05e-6 + 2.2e-8 * (double)n) + 0.0037 * item + 4.4e-4 * (double)p->m +
+               (reds > 0 ? 2.2 + 0.036 * reds : 0);
+    int64_t ln = 1;
+    while (ln < 32 && ln < vecs) ln *= 2;
+    const double nch = (double)((vecs + ln - 1) / ln);
+    return (f32 ? 2.18 : 2.3) + 2.3e-4 * (double)p->n_items * nch +
+           nnz * ((f32 ? 4.7e-7 : 3.0e-7) * (double)ln * nch +
+                  (double)n * (f32 ? 4 * 3.5e-8 : 2 * 1.75e-7)) +
+           item * (0.0015 * (double)ln + (f32 ? 0.0046 : 0.0042)) +
+           (reds > 0 ? 2.0 + 0.015 * reds * (double)((n + 127) / 128) : 0);
+}
+
+bool gather_xs_takes(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, const void *Y,
+                     int64_t ldy) {
+    if (!p->gx.on || n < 1) return false;
     int ln, cs;
-    const bool one = n == 1 || n == 2 || n == 4 || n == 8;
     if (p->xdt == SPMM_F32) {
+        // more than one vector per row, and a slice that holds as many columns
+        // as one warp covers
         int cover = 1;
         while (cover < 8 && cover * 4 < n) cover *= 2;
-        return n > 4 && gx_shape<float>(p, n, &ln, &cs) && ln == cover;
+        if (n <= 4 || !gx_shape<float>(p, n, &ln, &cs) || ln != cover) return false;
+    } else {
+        if (!gx_shape<__half>(p, n, &ln, &cs)) return false;
     }
-    return !(one && gather_ring_fits(p, n)) && gx_shape<__half>(p, n, &ln, &cs);
+    // one vector of X per row that fits the ring kernel's memory: that kernel
+    // (8192 x 8192, n = 1: 8.3 against 13.5 us)
+    if (gather_vector(p, X, n, ldx, Y, ldy) == n && gather_ring_fits(p, n)) return false;
+    return gx_us(p, X, n, ldx, ln, cs) < 0.85 * items_us(p, X, n, ldx, Y, ldy);
 }
 
 cudaError_t launch_gather_xs(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, void *Y,

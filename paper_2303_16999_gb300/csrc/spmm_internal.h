@@ -89,6 +89,15 @@ struct TcShape {
 TcShape choose_tc_shape(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
                         const int32_t *bcol, int64_t n, int sms, int ct_only, int default_rows);
 
+// b = 1 plans the X-in-shared-memory gather may run: how the non-zeros lie
+// over its CTAs and warps.  [c]: k cut into 2^c slices.
+struct GxLoad {
+    bool on = false;
+    int64_t longest_row = 0;       // non-zeros of a row
+    int64_t row_slice[3] = {};     // ... and of a row in one slice, at most
+    int64_t heavy[3][8] = {};      // non-zeros of the heaviest slice of 2^j equal row ranges
+};
+
 // ------------------------------------------------------------------- plan
 // dynamic plans: scratch of the device re-partition
 struct DynBufs {
@@ -139,6 +148,7 @@ struct spmm_plan {
     uint32_t *d_srec = nullptr, *d_sprog = nullptr;  // TC: stage records and MMA programs
     uint16_t *d_col16 = nullptr;   // static GATHER plans, k <= 65536: col_idx in 16 bits
     int32_t *d_gx_ptr = nullptr;   // with it: the first non-zero of every (row, part of k)
+    spmm::GxLoad gx;                     // what a launch of k_gather_xs.cu would find (host)
     // TC, batched with plans of the other stage geometry: this plan's stage
     // records cut for that geometry (built on first use), geometry alt_geo
     uint32_t *d_srec_alt = nullptr, *d_sprog_alt = nullptr;
@@ -200,10 +210,14 @@ cudaError_t launch_pack_tiles(const spmm_plan *p, const void *d_values, const fl
                               const int32_t *d_nnzb, cudaStream_t s);
 cudaError_t launch_plain(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
                          int64_t ldy, cudaStream_t s);
+// columns per load of the gather kernels on these operands
+int gather_vector(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, const void *Y,
+                  int64_t ldy);
 // whether X of n columns fits the gather ring kernel's shared memory
 bool gather_ring_fits(const spmm_plan *p, int64_t n);
-// b = 1 with X in shared memory (k_gather_xs.cu); whether it takes n columns
-bool gather_xs_takes(const spmm_plan *p, int64_t n);
+// b = 1 with X in shared memory (k_gather_xs.cu); whether it takes this call
+bool gather_xs_takes(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, const void *Y,
+                     int64_t ldy);
 cudaError_t launch_gather_xs(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
                              int64_t ldy, cudaStream_t s);
 // FP32 blocks, b >= 4 (k_f32.cu); launch_plain is the one-thread-per-output kernel

@@ -76,7 +76,7 @@ class PlanInfo(ctypes.Structure):
                                       "ws_rows", "n_reductions", "device_bytes")] + \
         [(n, ctypes.c_int32) for n in ("stage_geometry", "sddmm_form")] + \
         [(n, ctypes.c_int64) for n in ("row_begin", "row_end")] + \
-        [(n, ctypes.c_int32) for n in ("col_tiles", "index_bytes")]
+        [(n, ctypes.c_int32) for n in ("col_tiles", "index_bytes", "auto_col_tiles", "gather_form")]
 
 
 class TuneChoice(ctypes.Structure):
