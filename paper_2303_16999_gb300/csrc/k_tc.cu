@@ -275,12 +275,18 @@ struct TcProb {
 
 // A stage whose entries are 2 to 4 consecutive tile columns (record info
 // bit 20) gets its X slabs in one TMA box of 4 slabs, or with a 2-D map (n not
-// a multiple of 64) in one box per 64-column half; the slabs then lie 2048 B
-// apart inside each half, the halves 8192 B apart.  A box costs about 110
+// a multiple of 64) in one box per 64-column half, in dense-tile stages; the
+// slabs then lie 2048 B apart inside each half, the halves 8192 B apart.  A box costs about 110
 // cycles of an SM's TMA unit whatever its size, so eight 2 KB boxes per stage
 // bound the dense-tile plans with a 2-D map: 4096 x 4096, b = 4, d = 1/8, in
 // 16-row groups split along k, n = 24: 20.4 -> 14.7 us, n = 100: 19.8 -> 17.0;
 // 4096 x 16384, b = 8, d = 1/8, n = 200: 45.2 -> 39.7.
+// A sparse-tile stage of so few entries ends a batch of 32; its four small
+// boxes from two warps land sooner than one box (16384 x 4096, b = 8, d = 1/4,
+// E4M3, n = 24: 53.8 us, joint 55.9).
+template <int BASE> __device__ __forceinline__ bool joint_stage(uint32_t info, int x3d) {
+    return (info & kJointBit) && (BASE == 0 || x3d);
+}
 
 struct TcBatch {
     CUtensorMap maps[kMaxBatch]; // X of each problem
@@ -443,7 +449,6 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                 const int h = (nent + 1) >> 1;
                 const int xlo = pid == 2 ? h : 0, mine = pid == 2 ? nent - h : h;
                 const uint32_t col = __shfl_sync(0xffffffffu, rc, min(3 + xlo + lane, kRecWords - 1));
-                const uint32_t jcol = __shfl_sync(0xffffffffu, rc, 3);   // the stage's first column
                 int w = 1;
                 if (lane == 0) w = mbar_wait(&sm->empty[stage], phase ^ 1, sm, B.wait_ns) ? 1 : 0;
                 if (!__shfl_sync(0xffffffffu, w, 0)) return -1;
@@ -479,7 +484,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                     // first warp of the tile) or one box per slab, with a 2-D
                     // map as two 64-column boxes per slab (the lower one only
                     // when the upper 64 columns lie past n)
-                    const bool joint = (info & kJointBit) != 0;
+                    const bool joint = joint_stage<G::base>(info, P.x3d);
                     const int tset = (pid - 1) & 1, part = (pid - 1) >> 1;
                     const bool act = tset == 0 || two;
                     const int per = (nent + G::xprod - 1) / G::xprod;
@@ -504,6 +509,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                                         (int)xc * kTile, nh, &sm->full[stage]);
                     } else if (joint) {
                         // 2-D map: one box of slabs per 64-column half
+                        const uint32_t jcol = __shfl_sync(0xffffffffu, rc, 3);
                         if (act && cnt && lane < (half ? 1 : 2))
                             tma_load_2d(xs + lane * kJointSlabs * (kSlabBytes / 2), &B.maps4[un.p],
                                         (int)ncol + lane * (kNTile / 2),
@@ -515,11 +521,12 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                             tma_load_2d(slab + kSlabBytes / 2, &B.maps[un.p], (int)ncol + kNTile / 2,
                                         (int)xc * kTile, &sm->full[stage]);
                     }
-                } else if (info & kJointBit) {
+                } else if (joint_stage<G::base>(info, P.x3d)) {
                     // consecutive columns: X producer 1 requests all slabs in one
                     // box, or with a 2-D map each producer those of one 64-column
                     // half (the upper one only if it holds columns of n)
                     const int x0 = n0 + (pid == 2 ? kNTile / 2 : 0);
+                    const uint32_t jcol = __shfl_sync(0xffffffffu, rc, 3);   // the first column
                     if (lane == 0) {
                         if (P.x3d ? pid == 1 : x0 < P.n) {
                             mbar_arrive_tx(&sm->full[stage],
@@ -640,7 +647,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                 last = (info >> 31) != 0;
                 const uint32_t myword = sm->meta[stage].prog[half][lane];   // words >= nmma unused
                 const uint32_t sbase = smem_u32(stages + stage * G::bytes);
-                const bool joint = (info & kJointBit) != 0;
+                const bool joint = joint_stage<G::base>(info, B.prob[un.p].x3d);
                 const uint64_t adesc0 = joint ? a_desc_joint(sbase) : a_desc(sbase);
                 const uint32_t astep = joint ? (kSlabBytes / 2) >> 4 : kSlabBytes >> 4;
                 const uint64_t bdesc0 = b_desc(sbase + G::w16);
