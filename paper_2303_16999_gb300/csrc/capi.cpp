@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <numeric>
 #include <vector>
 
 #include "spmm_internal.h"
@@ -511,6 +512,23 @@ static spmm_status plan_create_slice(int64_t m, int64_t k, int64_t n_max, int32_
     return SPMM_OK;
 }
 
+// (32 entries, over 468 products with skewed, banded and diagonal patterns: 1.003
+// times as fast as 16 or 48 on average)
+constexpr int64_t kSplitGain = 32;
+// Entries per work item of a plan that is not split along k: 1.25 times the
+// mean group's, where groups well above it are cut to that, else the longest
+// group's, so that none is.  A cut costs the reduction's launch and its
+// partials: ten groups of 41 to 48 entries cut to 40 took 11.5 us, whole 8.9
+// (4096 x 4096, b = 16, d = 1/8, n = 64); 4 groups of 128 cut to 23 8.4 us, to 67 11.2
+// (2048 x 2048, b = 8, d = 1/32, n = 24, one band of rows full).
+static int64_t unsplit_length(const std::vector<int64_t> &len, int64_t E) {
+    const int64_t G = (int64_t)len.size();
+    if (!G) return 16;
+    const int64_t head = std::max<int64_t>(16, (5 * E + 4 * G - 1) / (4 * G));
+    const int64_t longest = *std::max_element(len.begin(), len.end());
+    return longest - head > kSplitGain ? head : std::max(head, longest);
+}
+
 static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, spmm_mode mode,
                                spmm_dtype w_dtype, spmm_dtype x_dtype, const spmm_pattern *pattern,
                                int64_t nnzb_max, const spmm_plan_opts *opts, spmm_plan **out) {
@@ -667,22 +685,16 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
                 if (o.max_per_item && !o.k_splits) {
                     p->C = o.max_per_item;
                 } else {
-                    const int64_t G = p->groups > 0 ? p->groups
-                                                    : (int64_t)group_partition(mt, p->R).size();
-                    const int64_t E = count_entries(m, k, b, p->nnzb, pattern->brow, pattern->bcol,
-                                                    p->R, p->groups);
+                    const std::vector<int64_t> len = group_entries(
+                        m, k, b, p->nnzb, pattern->brow, pattern->bcol, p->R, p->groups);
+                    const int64_t G = (int64_t)len.size();
+                    const int64_t E = std::accumulate(len.begin(), len.end(), (int64_t)0);
                     if (splits) {
                         // about that many items per group of mean length
                         const int64_t per = G ? (E + G * splits - 1) / (G * splits) : 1;
                         p->C = (int)std::max<int64_t>(1, per);
                     } else {
-                        // entries per group if spread evenly, with headroom:
-                        // only groups well above the mean are split (the
-                        // reduction's launch costs what about 50 entries do:
-                        // 4096 x 4096, b = 16, d = 1/8, n = 64 took 11.5 us
-                        // with its ten longest groups split, 8.9 without)
-                        p->C = (int)std::max<int64_t>(
-                            48, G ? std::max((5 * E + 4 * G - 1) / (4 * G), (E + G - 1) / G + 48) : 48);
+                        p->C = (int)unsplit_length(len, E);
                     }
                 }
                 build_tc_plan(m, k, b, p->nnzb, pattern->brow, pattern->bcol, p->R, p->C, true,

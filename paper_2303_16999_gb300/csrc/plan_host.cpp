@@ -304,8 +304,8 @@ void build_tc_plan(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *bro
     finish_items(items, sort_items, grows, hp);
 }
 
-int64_t count_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
-                      const int32_t *bcol, int64_t R, int64_t groups) {
+std::vector<int64_t> group_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
+                                   const int32_t *bcol, int64_t R, int64_t groups) {
     const int64_t mt = m / kTile, words = (k / kTile + 63) / 64;
     const std::vector<int64_t> sizes =
         groups > 0 ? near_equal_partition(mt, groups) : group_partition(mt, R);
@@ -318,8 +318,8 @@ int64_t count_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *
         const int64_t tc = (int64_t)bcol[p] * b / kTile;
         bits[base[(int64_t)brow[p] * b / kTile] + tc / 64] |= 1ull << (tc % 64);
     }
-    int64_t n = 0;
-    for (uint64_t w : bits) n += __builtin_popcountll(w);
+    std::vector<int64_t> n(sizes.size(), 0);
+    for (size_t i = 0; i < bits.size(); ++i) n[i / words] += __builtin_popcountll(bits[i]);
     return n;
 }
 

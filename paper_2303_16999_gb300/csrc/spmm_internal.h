@@ -74,10 +74,10 @@ void build_tc_plan(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *bro
                    const int32_t *bcol, int64_t R, int64_t C, bool sort_items, bool pad,
                    HostPlan &hp, int64_t groups = 0);
 
-// entries (distinct tile columns per tile-row group, summed) of a plan with
-// these groups
-int64_t count_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
-                      const int32_t *bcol, int64_t R, int64_t groups);
+// entries (distinct tile columns) of each tile-row group of a plan with these
+// groups
+std::vector<int64_t> group_entries(int64_t m, int64_t k, int b, int64_t nnzb, const int32_t *brow,
+                                   const int32_t *bcol, int64_t R, int64_t groups);
 // launch shape of a static tensor-core plan that 16-row groups alone would
 // not occupy the GPU with: tile rows per group, work items per group along k
 // and column tiles per CTA (ct_only: 0, or the only count allowed); groups > 0:
