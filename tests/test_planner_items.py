@@ -54,3 +54,26 @@ def test_a_full_band_is_cut():
     length = np.diff(p.array("grp_ebeg"))
     assert length.max() == 128 and (items[:, 2] - items[:, 1]).max() <= 32
     assert p.info()["n_reductions"] >= 4
+
+
+def test_automatic_splits_stay_in_one_wave():
+    """Plans that the planner splits along k make no more units (items x
+    column tiles) than run at once on 152 SMs: two per SM, or one that covers
+    two column tiles."""
+    rng = np.random.default_rng(5)
+    split = 0
+    sizes = [(624, 9056, 45, 8, 16), (592, 3936, 217, 4, 32), (1952, 3024, 51, 4, 16),
+             (976, 3568, 120, 8, 8), (640, 15888, 122, 8, 8), (384, 7936, 245, 4, 32),
+             (272, 10640, 66, 8, 8), (1936, 15120, 25, 16, 8), (256, 6160, 147, 4, 16),
+             (672, 10592, 369, 4, 64), (608, 14112, 70, 16, 8)]
+    sizes += [(16 * int(2 ** rng.uniform(4, 7)), 16 * int(2 ** rng.uniform(6, 9.5)),
+               int(2 ** rng.uniform(4, 9)), int(rng.choice([4, 8, 16])),
+               int(rng.choice([8, 16, 32]))) for _ in range(60)]
+    for m, k, n, b, d in sizes:
+        i = _plan(_mask(rng, m // b, k // b, "uniform", 1 / d), b, n).info()
+        if i["n_items"] < 1.9 * i["n_groups"]:
+            continue
+        split += 1
+        cols, slots = (256, 152) if i["auto_col_tiles"] == 2 else (128, 304)
+        assert i["n_items"] * -(-n // cols) <= slots, (m, k, n, b, d, i)
+    assert split >= 30
