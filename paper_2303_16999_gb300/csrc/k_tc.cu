@@ -283,7 +283,8 @@ struct TcProb {
 // 4096 x 16384, b = 8, d = 1/8, n = 200: 45.2 -> 39.7.
 // A sparse-tile stage of so few entries ends a batch of 32; its four small
 // boxes from two warps land sooner than one box (16384 x 4096, b = 8, d = 1/4,
-// E4M3, n = 24: 53.8 us, joint 55.9).
+// E4M3, n = 24: 53.8 us, joint 55.9), and without that code their launches of 5 to
+// 10 us take 1 % less.
 template <int BASE> __device__ __forceinline__ bool joint_stage(uint32_t info, int x3d) {
     return (info & kJointBit) && (BASE == 0 || x3d);
 }
@@ -507,7 +508,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                         if (act && !joint && lane < cnt)
                             tma_load_3d(xs + (lo + lane) * kSlabBytes, &B.maps[un.p], 0,
                                         (int)xc * kTile, nh, &sm->full[stage]);
-                    } else if (joint) {
+                    } else if (G::base == 0 && joint) {
                         // 2-D map: one box of slabs per 64-column half
                         const uint32_t jcol = __shfl_sync(0xffffffffu, rc, 3);
                         if (act && cnt && lane < (half ? 1 : 2))
@@ -526,12 +527,13 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                     // box, or with a 2-D map each producer those of one 64-column
                     // half (the upper one only if it holds columns of n)
                     const int x0 = n0 + (pid == 2 ? kNTile / 2 : 0);
+                    const bool d3 = G::base != 0 || P.x3d;   // (as joint_stage)
                     const uint32_t jcol = __shfl_sync(0xffffffffu, rc, 3);   // the first column
                     if (lane == 0) {
-                        if (P.x3d ? pid == 1 : x0 < P.n) {
+                        if (d3 ? pid == 1 : x0 < P.n) {
                             mbar_arrive_tx(&sm->full[stage],
-                                           kJointSlabs * (P.x3d ? kSlabBytes : kSlabBytes / 2));
-                            if (P.x3d)
+                                           kJointSlabs * (d3 ? kSlabBytes : kSlabBytes / 2));
+                            if (d3)
                                 tma_load_3d(st, &B.maps4[un.p], 0, (int)jcol * kTile,
                                             n0 / (kNTile / 2), &sm->full[stage]);
                             else
