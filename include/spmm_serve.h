@@ -6,10 +6,11 @@
  *
  * Model: requests queue in arrival order.  A request is admitted when its
  * device staging (X_r and Y_r, 16-bit) fits the HBM budget; admitted
- * requests of any mix of weights are launched together in one persistent
- * tensor-core launch on one of up to max_inflight streams ("slots"), so
- * requests that arrive while others run are admitted as slots and budget
- * free up and their work overlaps on the device (continuous batching).
+ * requests of any mix of weights with the same W and X types are launched
+ * together in one persistent tensor-core launch on one of up to max_inflight
+ * streams ("slots"), so requests that arrive while others run are admitted as
+ * slots and budget free up and their work overlaps on the device (continuous
+ * batching).
  * Y_r is copied back to the caller's host buffer when its launch finishes.
  * Column j of Y depends only on column j of X, and the work order of a
  * column does not depend on its neighbours, so a result is the same alone

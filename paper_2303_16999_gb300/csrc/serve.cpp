@@ -165,6 +165,11 @@ void serve_server::batcher_loop() {
             spmm_plan *p = weights[r.w];
             const bool b = batchable(p);
             if (!L.reqs.empty() && (!b || !tc)) break;
+            // a launch has one kernel, for one pair of W and X types
+            if (!L.reqs.empty()) {
+                const spmm_plan *q = weights[reqs[L.reqs[0]].w];
+                if (p->wdt != q->wdt || p->xdt != q->xdt) break;
+            }
             if ((int)L.reqs.size() >= cfg.max_batch || cols + r.n > cfg.max_batch_n) break;
             // a weight with split rows (shared workspace) or a non-batched
             // weight runs in one launch at a time, once per launch

@@ -1,5 +1,5 @@
-"""Serving weights that differ in stage geometry, on several launches in
-flight at a time.  Operands are integer-valued, so every Y must equal the
+"""Serving weights that differ in stage geometry and in type, on several
+launches in flight at a time.  Operands are integer-valued, so every Y must equal the
 64-bit product rounded once, whatever shares a launch with it.
 """
 import pytest
@@ -68,3 +68,22 @@ def test_both_geometries_on_four_launches():
         for w in ws:
             assert w["plan"].status() == 0
             w["plan"].close()
+
+
+def test_types_do_not_share_a_launch():
+    """F16, BF16 and E4M3 weights in one queue, all of it there before the
+    second launch: neighbours of one type may share one, others never do."""
+    ws = [_weight(200 + i, 256, 512, 64, 8, 1 / 4, wt=t)
+          for i, t in enumerate(("f16", "bf16", "e4m3", "f16"))]
+    torch.cuda.synchronize()
+    srv = S.Server(hbm_budget_bytes=64 << 20, max_inflight=2, inject_delay_us=100000)
+    ids = [srv.register(w["plan"]) for w in ws]
+    seq = [0, 0, 1, 2, 2, 1, 3, 0, 2, 0]
+    _serve(srv, _requests(ws, ids, [(i, 5 + 6 * q) for q, i in enumerate(seq)]))
+    st = srv.stats()
+    srv.close()
+    assert st["completed"] == len(seq) and st["failed"] == 0
+    assert st["launches"] >= 7        # runs of one type: 0 0 | 1 | 2 2 | 1 | 3 0 | 2 | 0
+    for w in ws:
+        assert w["plan"].status() == 0
+        w["plan"].close()
