@@ -11,6 +11,9 @@
  * streams ("slots"), so requests that arrive while others run are admitted as
  * slots and budget free up and their work overlaps on the device (continuous
  * batching).
+ * Weights whose plans split rows keep one set of partial sums in the plan; a
+ * request to such a weight while another holds it takes its partials (FP32,
+ * ws_rows x n of the plan's info) from the same budget, or waits.
  * Y_r is copied back to the caller's host buffer when its launch finishes.
  * Column j of Y depends only on column j of X, and the work order of a
  * column does not depend on its neighbours, so a result is the same alone
@@ -34,7 +37,7 @@ extern "C" {
 typedef struct serve_server serve_server;
 
 typedef struct {
-    int64_t hbm_budget_bytes;  /* device bytes for request staging (X_r + Y_r); > 0 */
+    int64_t hbm_budget_bytes;  /* device bytes for request staging (X_r + Y_r, partials); > 0 */
     int32_t max_inflight;      /* concurrent launches (streams), 1..8 */
     int32_t max_batch;         /* requests per launch, 1..64 */
     int64_t max_batch_n;       /* total columns per launch, >= 1 */

@@ -833,7 +833,8 @@ cudaError_t launch_gather(const spmm_plan *p, const void *X, int64_t n, int64_t 
 }
 
 cudaError_t launch_reduce_tc(int count, const spmm_plan *const *plans, const int64_t *n,
-                             void *const *Y, const int64_t *ldy, cudaStream_t s) {
+                             void *const *Y, const int64_t *ldy, cudaStream_t s,
+                             float *const *ws) {
     RedBatch B;
     B.nprob = 0;
     int64_t reds = 0, most = 0;
@@ -843,8 +844,9 @@ cudaError_t launch_reduce_tc(int count, const spmm_plan *const *plans, const int
         if (p->n_red == 0 || n[i] == 0) continue;
         const int64_t ly = ldy ? ldy[i] : n[i];
         const int yvec = n[i] % 4 == 0 && ly % 4 == 0 && (uintptr_t)Y[i] % 8 == 0;
-        B.prob[B.nprob++] = RedProb{p->d_red, p->d_grp_row0, p->d_grp_rows, p->d_ws, p->d_ws_row0,
-                                    Y[i], ly, (int32_t)n[i], (int32_t)reds, yvec};
+        B.prob[B.nprob++] = RedProb{p->d_red, p->d_grp_row0, p->d_grp_rows,
+                                    ws && ws[i] ? ws[i] : p->d_ws, p->d_ws_row0, Y[i], ly,
+                                    (int32_t)n[i], (int32_t)reds, yvec};
         reds += p->n_red;
         most = std::max(most, (int64_t)p->R * kTile * n[i] / 4);
         any = p;
@@ -852,7 +854,8 @@ cudaError_t launch_reduce_tc(int count, const spmm_plan *const *plans, const int
     if (!any) return cudaSuccess;
     if (reds > 65535) {   // the grid's y limit
         for (int i = 0; i < count; ++i) {
-            const cudaError_t e = launch_reduce(plans[i], n[i], Y[i], ldy ? ldy[i] : n[i], s);
+            const cudaError_t e = launch_reduce(plans[i], n[i], Y[i], ldy ? ldy[i] : n[i], s,
+                                                ws ? ws[i] : nullptr);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;
@@ -866,7 +869,9 @@ cudaError_t launch_reduce_tc(int count, const spmm_plan *const *plans, const int
     return pdl_launch(reduce_tc_kernel<__half>, grid, dim3(kRedThreads), 0, s, B);
 }
 
-cudaError_t launch_reduce(const spmm_plan *p, int64_t n, void *Y, int64_t ldy, cudaStream_t s) {
+cudaError_t launch_reduce(const spmm_plan *p, int64_t n, void *Y, int64_t ldy, cudaStream_t s,
+                          const float *ws) {
+    if (!ws) ws = p->d_ws;
     const bool dyn = p->mode == SPMM_DYNAMIC;
     const int64_t n_red = dyn ? p->dyn.red_cap : p->n_red;
     const int32_t *n_red_dev = dyn ? p->d_counts + kCntRed : nullptr;
@@ -891,17 +896,17 @@ cudaError_t launch_reduce(const spmm_plan *p, int64_t n, void *Y, int64_t ldy, c
     switch (p->xdt) {
         case SPMM_F32:
             pdl_launch(reduce_kernel<float>, dim3(grid), dim3(128), 0, s, p->d_red, r0, rn,
-                rows_per_unit, p->d_ws, p->d_ws_row0, (float *)Y, ldy, n, n_red, n_red_dev,
+                rows_per_unit, ws, p->d_ws_row0, (float *)Y, ldy, n, n_red, n_red_dev,
                 p->d_status, bar);
             break;
         case SPMM_F16:
             pdl_launch(reduce_kernel<__half>, dim3(grid), dim3(128), 0, s, p->d_red, r0, rn,
-                rows_per_unit, p->d_ws, p->d_ws_row0, (__half *)Y, ldy, n, n_red, n_red_dev,
+                rows_per_unit, ws, p->d_ws_row0, (__half *)Y, ldy, n, n_red, n_red_dev,
                 p->d_status, bar);
             break;
         case SPMM_BF16:
             pdl_launch(reduce_kernel<__nv_bfloat16>, dim3(grid), dim3(128), 0, s, p->d_red, r0, rn,
-                rows_per_unit, p->d_ws, p->d_ws_row0, (__nv_bfloat16 *)Y, ldy, n, n_red, n_red_dev,
+                rows_per_unit, ws, p->d_ws_row0, (__nv_bfloat16 *)Y, ldy, n, n_red, n_red_dev,
                 p->d_status, bar);
             break;
         default: return cudaErrorInvalidValue;

@@ -988,8 +988,9 @@ bool use_deep(const spmm_plan *p, int64_t units) {
     return p->mode == SPMM_STATIC && units <= p->sm_count;
 }
 
+// ws: the launch's partials of split groups, if not in the plan's own workspace
 void fill_prob(TcProb &P, const spmm_plan *p, void *Y, int64_t n, int64_t ldy, int x3d,
-               bool alt = false) {
+               bool alt = false, float *ws = nullptr) {
     P.items = p->d_items;
     P.grp_row0 = p->d_grp_row0;
     P.grp_rows = p->d_grp_rows;
@@ -999,7 +1000,7 @@ void fill_prob(TcProb &P, const spmm_plan *p, void *Y, int64_t n, int64_t ldy, i
     P.packed = (const uint8_t *)p->d_packed;
     P.tile_scale = p->d_tile_scale;
     P.Y = Y;
-    P.ws = p->d_ws;
+    P.ws = ws ? ws : p->d_ws;
     P.ws_row0 = p->d_ws_row0;
     P.srec = alt ? p->d_srec_alt : p->d_srec;
     P.sprog = alt ? p->d_sprog_alt : p->d_sprog;
@@ -1127,7 +1128,8 @@ cudaError_t launch_tc(const spmm_plan *p, const void *X, int64_t n, int64_t ldx,
 namespace {
 cudaError_t launch_tc_group(int count, spmm_plan *const *plans, const void *const *X,
                             const int64_t *n, const int64_t *ldx, void *const *Y,
-                            const int64_t *ldy, cudaStream_t s, bool schedule, int geo);
+                            const int64_t *ldy, cudaStream_t s, bool schedule, int geo,
+                            float *const *ws);
 cudaError_t ensure_alt_records(spmm_plan *p, int geo);
 }
 
@@ -1139,13 +1141,15 @@ cudaError_t ensure_alt_records(spmm_plan *p, int geo);
 // n > 128) run in a second launch of the two-column-tile kernel.
 cudaError_t launch_tc_batch(int count, spmm_plan *const *plans, const void *const *X,
                             const int64_t *n, const int64_t *ldx, void *const *Y,
-                            const int64_t *ldy, cudaStream_t s, bool schedule) {
+                            const int64_t *ldy, cudaStream_t s, bool schedule,
+                            float *const *ws) {
     if (count <= 0 || count > kMaxBatch) return cudaErrorInvalidValue;
     for (int wide = 0; wide < 2; ++wide) {
         spmm_plan *gp[kMaxBatch];
         const void *gx[kMaxBatch];
         void *gy[kMaxBatch];
         int64_t gn[kMaxBatch], glx[kMaxBatch], gly[kMaxBatch];
+        float *gw[kMaxBatch];
         int c = 0;
         int64_t units[2] = {0, 0};
         for (int i = 0; i < count; ++i) {
@@ -1154,6 +1158,7 @@ cudaError_t launch_tc_batch(int count, spmm_plan *const *plans, const void *cons
             gp[c] = plans[i];
             gx[c] = X[i];
             gy[c] = Y[i];
+            gw[c] = ws ? ws[i] : nullptr;
             gn[c] = n[i];
             glx[c] = ldx ? ldx[i] : n[i];
             gly[c] = ldy ? ldy[i] : n[i];
@@ -1167,7 +1172,7 @@ cudaError_t launch_tc_batch(int count, spmm_plan *const *plans, const void *cons
             cudaError_t e = ensure_alt_records(gp[i], geo);
             if (e != cudaSuccess) return e;
         }
-        cudaError_t e = launch_tc_group(c, gp, gx, gn, glx, gy, gly, s, schedule, geo + 2 * wide);
+        cudaError_t e = launch_tc_group(c, gp, gx, gn, glx, gy, gly, s, schedule, geo + 2 * wide, gw);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1220,7 +1225,8 @@ cudaError_t ensure_alt_records(spmm_plan *p, int geo) {
 
 cudaError_t launch_tc_group(int count, spmm_plan *const *plans, const void *const *X,
                             const int64_t *n, const int64_t *ldx, void *const *Y,
-                            const int64_t *ldy, cudaStream_t s, bool schedule, int geo) {
+                            const int64_t *ldy, cudaStream_t s, bool schedule, int geo,
+                            float *const *ws) {
     TcBatch B;
     std::lock_guard<std::mutex> lk(g_sched_mu);
     SchedKey key;
@@ -1235,7 +1241,7 @@ cudaError_t launch_tc_group(int count, spmm_plan *const *plans, const void *cons
             e = encode_x(&B.maps4[i], &x3d, p->xdt == SPMM_BF16, X[i], p->k, n[i], lx,
                          kJointSlabs);
         if (e != cudaSuccess) return e;
-        fill_prob(B.prob[i], p, Y[i], n[i], ly, x3d, p->tc_geo != (geo & 1));
+        fill_prob(B.prob[i], p, Y[i], n[i], ly, x3d, p->tc_geo != (geo & 1), ws[i]);
         if (geo >= 2) B.prob[i].ntn = (B.prob[i].ntn + 1) / 2;   // units of two column tiles
         B.prob[i].unit_base = base;
         base += p->n_items * B.prob[i].ntn;

@@ -79,6 +79,9 @@ struct Req {
     ReqState state = kQueued;
     spmm_status st = SPMM_OK;
     int64_t xoff = -1, yoff = -1, xbytes = 0, ybytes = 0;
+    // a split weight's partials in the staging pool (woff < 0: in the plan's
+    // own workspace)
+    int64_t woff = -1, wbytes = 0;
 };
 
 struct Launch {
@@ -118,6 +121,11 @@ struct serve_server {
     int64_t submitted = 0, admitted = 0, completed = 0, rejected = 0, failed = 0, launches = 0;
     double sum_reqs = 0, sum_cols = 0, first_arr = -1, last_done = -1, flops_done = 0;
 
+    void release(const Req &r) {
+        pool.release(r.xoff, r.xbytes);
+        pool.release(r.yoff, r.ybytes);
+        if (r.woff >= 0) pool.release(r.woff, r.wbytes);
+    }
     void fail_locked(uint64_t id, spmm_status st) {
         Req &r = reqs[id];
         r.state = kDone;
@@ -171,15 +179,11 @@ void serve_server::batcher_loop() {
                 if (p->wdt != q->wdt || p->xdt != q->xdt) break;
             }
             if ((int)L.reqs.size() >= cfg.max_batch || cols + r.n > cfg.max_batch_n) break;
-            // a weight with split rows (shared workspace) or a non-batched
-            // weight runs in one launch at a time, once per launch
-            const bool exclusive = !b || p->n_red > 0;
-            if (exclusive) {
-                if (weight_busy[r.w]) break;
-                bool dup = false;
-                for (uint64_t o : L.reqs) dup |= reqs[o].w == r.w;
-                if (dup) break;
-            }
+            // a non-batched weight runs in one launch at a time, once per
+            // launch; so does a plan's workspace, which one request at a time
+            // to a weight with split rows takes: others bring their own
+            const bool own = !b || (p->n_red > 0 && !weight_busy[r.w]);
+            if (!b && weight_busy[r.w]) break;
             if (cfg.inject_alloc_fail) {
                 queue.pop_front();
                 fail_locked(id, SPMM_ERR_OOM);
@@ -192,14 +196,21 @@ void serve_server::batcher_loop() {
                 pool.release(xo, r.xbytes);
                 break;
             }
+            int64_t wo = -1;
+            if (b && p->n_red > 0 && !own && !pool.alloc(r.wbytes, &wo)) {
+                pool.release(xo, r.xbytes);
+                pool.release(yo, r.ybytes);
+                break;
+            }
             r.xoff = xo;
             r.yoff = yo;
+            r.woff = wo;
             queue.pop_front();
             L.reqs.push_back(id);
             cols += r.n;
             tc = b;
             ++admitted;
-            if (exclusive) {
+            if (own) {
                 L.busy_weights.push_back(r.w);
                 weight_busy[r.w] = 1;
             }
@@ -219,6 +230,7 @@ void serve_server::batcher_loop() {
         std::vector<int64_t> ns(cnt), lxs(cnt), lys(cnt);
         std::vector<const void *> hx(cnt);
         std::vector<void *> hy(cnt);
+        std::vector<float *> ws(cnt);
         for (int i = 0; i < cnt; ++i) {
             Req &r = reqs[L.reqs[i]];
             r.state = kLaunched;
@@ -230,6 +242,7 @@ void serve_server::batcher_loop() {
             lys[i] = r.n;
             hx[i] = r.hX;
             hy[i] = r.hY;
+            ws[i] = r.woff < 0 ? nullptr : (float *)(pool_base + r.woff);
         }
         lk.unlock();
         if (cfg.inject_delay_us > 0)
@@ -258,9 +271,10 @@ void serve_server::batcher_loop() {
         if (e == cudaSuccess) {
             if (tc) {
                 e = launch_tc_batch(cnt, plans.data(), xs.data(), ns.data(), lxs.data(), ys.data(),
-                                    lys.data(), s, false);
+                                    lys.data(), s, false, ws.data());
                 if (e == cudaSuccess)
-                    e = launch_reduce_tc(cnt, plans.data(), ns.data(), ys.data(), lys.data(), s);
+                    e = launch_reduce_tc(cnt, plans.data(), ns.data(), ys.data(), lys.data(), s,
+                                         ws.data());
             } else {
                 spmm_status st = spmm_run(plans[0], nullptr, nullptr, nullptr, xs[0], ns[0],
                                           lxs[0], ys[0], lys[0], s);
@@ -281,8 +295,7 @@ void serve_server::batcher_loop() {
             cudaStreamSynchronize(s);
             for (uint64_t id : L.reqs) {
                 Req &r = reqs[id];
-                pool.release(r.xoff, r.xbytes);
-                pool.release(r.yoff, r.ybytes);
+                release(r);
                 fail_locked(id, SPMM_ERR_CUDA);
             }
             for (int32_t w : L.busy_weights) weight_busy[w] = 0;
@@ -321,8 +334,7 @@ void serve_server::completer_loop() {
                 const spmm_plan *p = weights[r.w];
                 r.state = kDone;
                 r.t_done = t;
-                pool.release(r.xoff, r.xbytes);
-                pool.release(r.yoff, r.ybytes);
+                release(r);
                 lat.push_back(t - r.t_arr);
                 ++completed;
                 flops_done += 2.0 * (double)p->nnzb * p->b * p->b * (double)r.n;
@@ -422,6 +434,7 @@ spmm_status serve_submit(serve_server *s, int32_t w, const void *h_X, int64_t n,
     const size_t es = es_of(p);
     r.xbytes = p->k * r.ldx * (int64_t)es;
     r.ybytes = p->m * n * (int64_t)es;
+    r.wbytes = p->hp.ws_rows * n * (int64_t)sizeof(float);
     if ((r.xbytes + 255) / 256 * 256 + (r.ybytes + 255) / 256 * 256 > s->cfg.hbm_budget_bytes) {
         ++s->rejected;
         set_error("serve_submit: request needs %lld staging bytes, budget is %lld",

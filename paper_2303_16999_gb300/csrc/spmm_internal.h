@@ -240,13 +240,18 @@ int tc_geometry(double tiles_per_entry);
 int64_t stage_prog_words();
 cudaError_t launch_tc(const spmm_plan *p, const void *d_X, int64_t n, int64_t ldx, void *d_Y,
                       int64_t ldy, cudaStream_t s);
-// the split groups of several static TC plans (16-bit outputs) in one launch
+// the split groups of several static TC plans (16-bit outputs) in one launch;
+// ws: each product's partials, where not in its plan's own workspace (NULL: all
+// there)
 cudaError_t launch_reduce_tc(int count, const spmm_plan *const *plans, const int64_t *n,
-                             void *const *Y, const int64_t *ldy, cudaStream_t s);
-cudaError_t launch_reduce(const spmm_plan *p, int64_t n, void *d_Y, int64_t ldy, cudaStream_t s);
+                             void *const *Y, const int64_t *ldy, cudaStream_t s,
+                             float *const *ws = nullptr);
+cudaError_t launch_reduce(const spmm_plan *p, int64_t n, void *d_Y, int64_t ldy, cudaStream_t s,
+                          const float *ws = nullptr);
 cudaError_t launch_tc_batch(int count, spmm_plan *const *plans, const void *const *X,
                             const int64_t *n, const int64_t *ldx, void *const *Y,
-                            const int64_t *ldy, cudaStream_t s, bool schedule);
+                            const int64_t *ldy, cudaStream_t s, bool schedule,
+                            float *const *ws = nullptr);
 // drops the cached batch schedules that name this plan
 void forget_schedules(const spmm_plan *p);
 cudaError_t launch_quantize_e4m3(int64_t nnzb, int b, spmm_dtype src, const void *d_src,

@@ -1,4 +1,5 @@
-"""Serving weights that differ in stage geometry and in type, on several
+"""Serving weights that differ in stage geometry, in type and in whether their
+plans split rows, on several
 launches in flight at a time.  Operands are integer-valued, so every Y must equal the
 64-bit product rounded once, whatever shares a launch with it.
 """
@@ -87,3 +88,51 @@ def test_types_do_not_share_a_launch():
     for w in ws:
         assert w["plan"].status() == 0
         w["plan"].close()
+
+
+def _split_weight(seed):
+    """A wide weight that the planner splits along k."""
+    w = _weight(seed, 512, 4096, 64, 8, 1 / 8)
+    assert w["plan"].info()["n_reductions"] > 0
+    return w
+
+
+def test_burst_to_a_split_weight_is_one_launch():
+    """The first request goes out alone; the others are all there when the
+    next launch is made, and share it."""
+    ws = [_split_weight(300), _weight(301, 512, 512, 64, 8, 1 / 4)]
+    torch.cuda.synchronize()
+    srv = S.Server(hbm_budget_bytes=256 << 20, max_inflight=2, inject_delay_us=100000)
+    ids = [srv.register(w["plan"]) for w in ws]
+    _serve(srv, _requests(ws, ids, [(1 if q % 5 == 3 else 0, 1 + 3 * q) for q in range(17)]))
+    st = srv.stats()
+    srv.close()
+    assert st["failed"] == 0 and st["launches"] == 2
+    assert all(w["plan"].status() == 0 for w in ws)
+
+
+def test_split_weight_on_four_launches():
+    """Launches of two requests, four in flight, all to one split weight and
+    one other: each has partials of its own."""
+    ws = [_split_weight(310), _weight(311, 512, 1024, 64, 8, 1 / 4)]
+    torch.cuda.synchronize()
+    srv = S.Server(hbm_budget_bytes=256 << 20, max_inflight=4, max_batch=2)
+    ids = [srv.register(w["plan"]) for w in ws]
+    for rnd in range(4):
+        _serve(srv, _requests(ws, ids, [(int(q % 3 == rnd), 1 + (7 * q + rnd) % 64)
+                                        for q in range(32)]))
+    assert srv.stats()["failed"] == 0
+    srv.close()
+    assert all(w["plan"].status() == 0 for w in ws)
+
+
+def test_split_weight_on_a_small_budget():
+    """A budget of one request's X and Y: partials fit nowhere but in the
+    plan, and requests follow one another."""
+    ws = [_split_weight(320)]
+    torch.cuda.synchronize()
+    srv = S.Server(hbm_budget_bytes=(4096 + 512) * 64 * 2, max_inflight=4)
+    ids = [srv.register(w["plan"]) for w in ws]
+    _serve(srv, _requests(ws, ids, [(0, n) for n in (64, 8, 40, 64, 3, 64, 64)]))
+    assert srv.stats()["failed"] == 0
+    srv.close()
