@@ -105,6 +105,7 @@ struct serve_server {
     Pool pool;
     std::vector<spmm_plan *> weights;
     std::vector<int> weight_busy;
+    std::vector<int32_t> home;   // the first id of a weight's plan: its workspace's owner
     std::mutex mu;
     std::condition_variable cv_batcher, cv_done;
     std::deque<uint64_t> queue;
@@ -182,8 +183,9 @@ void serve_server::batcher_loop() {
             // a non-batched weight runs in one launch at a time, once per
             // launch; so does a plan's workspace, which one request at a time
             // to a weight with split rows takes: others bring their own
-            const bool own = !b || (p->n_red > 0 && !weight_busy[r.w]);
-            if (!b && weight_busy[r.w]) break;
+            const int32_t w = home[r.w];
+            const bool own = !b || (p->n_red > 0 && !weight_busy[w]);
+            if (!b && weight_busy[w]) break;
             if (cfg.inject_alloc_fail) {
                 queue.pop_front();
                 fail_locked(id, SPMM_ERR_OOM);
@@ -211,8 +213,8 @@ void serve_server::batcher_loop() {
             tc = b;
             ++admitted;
             if (own) {
-                L.busy_weights.push_back(r.w);
-                weight_busy[r.w] = 1;
+                L.busy_weights.push_back(w);
+                weight_busy[w] = 1;
             }
             if (!b) break;  // non-batched weights: one request per launch
         }
@@ -404,6 +406,8 @@ spmm_status serve_register_weight(serve_server *s, spmm_plan *p, int32_t *weight
     }
     std::lock_guard<std::mutex> lk(s->mu);
     *weight_id = (int32_t)s->weights.size();
+    s->home.push_back((int32_t)(std::find(s->weights.begin(), s->weights.end(), p) -
+                                s->weights.begin()));
     s->weights.push_back(p);
     s->weight_busy.push_back(0);
     return SPMM_OK;

@@ -136,3 +136,17 @@ def test_split_weight_on_a_small_budget():
     _serve(srv, _requests(ws, ids, [(0, n) for n in (64, 8, 40, 64, 3, 64, 64)]))
     assert srv.stats()["failed"] == 0
     srv.close()
+
+
+def test_a_plan_under_two_ids():
+    """One split plan registered twice has one workspace: requests to both
+    ids, four launches in flight."""
+    ws = [_split_weight(330)] * 2
+    torch.cuda.synchronize()
+    srv = S.Server(hbm_budget_bytes=256 << 20, max_inflight=4, max_batch=1)
+    ids = [srv.register(w["plan"]) for w in ws]
+    for rnd in range(4):
+        _serve(srv, _requests(ws, ids, [(q % 2, 1 + (5 * q + rnd) % 64) for q in range(24)]))
+    assert srv.stats()["failed"] == 0
+    srv.close()
+    assert ws[0]["plan"].status() == 0
