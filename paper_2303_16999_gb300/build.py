@@ -6,7 +6,9 @@ front end; translation units compile in parallel and are linked into one
 shared library exporting the C ABI of ``include/spmm.h``.
 """
 import concurrent.futures as cf
+import hashlib
 import os
+import platform
 import subprocess
 import sys
 
@@ -29,41 +31,74 @@ def sources():
                   if f.endswith((".cu", ".cpp")))
 
 
-def _compile(src, extra):
-    obj = os.path.join(OUT_DIR, os.path.basename(src) + ".o")
-    headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
-    inc = os.path.join(ROOT, "include")
-    headers += [os.path.join(inc, f) for f in os.listdir(inc) if f.endswith(".h")]
-    newest = max(os.path.getmtime(p) for p in [src] + headers)
-    if os.path.exists(obj) and os.path.getmtime(obj) >= newest and not extra:
-        return obj
+def _flags(src, extra):
     lang = ["-x", "cu"] if src.endswith(".cu") else ["-x", "c++"]
-    cmd = [NVCC] + ARCH + COMMON + PER_FILE.get(os.path.basename(src), []) + list(extra) + lang + \
-        ["-c", src, "-o", obj]
-    r = subprocess.run(cmd, capture_output=True, text=True)
+    return ARCH + COMMON + PER_FILE.get(os.path.basename(src), []) + list(extra) + lang
+
+
+def _header_bytes():
+    inc = os.path.join(ROOT, "include")
+    paths = [os.path.join(d, f) for d in (CSRC, inc) for f in sorted(os.listdir(d))
+             if f.endswith((".h", ".cuh"))]
+    return b"".join(os.path.basename(p).encode() + open(p, "rb").read() for p in paths)
+
+
+def _key(*parts):
+    h = hashlib.sha256(platform.machine().encode())
+    for p in parts:
+        h.update(b"\0" + (p if isinstance(p, bytes) else p.encode()))
+    return h.hexdigest()
+
+
+def _fresh(path, key):
+    """Whether ``path`` was built from what ``key`` stands for."""
+    try:
+        return os.path.exists(path) and open(path + ".key").read() == key
+    except OSError:
+        return False
+
+
+def _run(cmd, out, key):
+    """Runs a build command that writes to a name beside ``out``, then puts
+    the result and its key in place."""
+    tmp = out + ".tmp%d" % os.getpid()
+    r = subprocess.run(cmd + ["-o", tmp], capture_output=True, text=True)
     if r.returncode != 0:
-        raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, " ".join(cmd), r.stderr))
+        raise RuntimeError("nvcc failed:\n%s\n%s" % (" ".join(cmd), r.stderr))
     if r.stderr.strip():
         sys.stderr.write(r.stderr)
-    return obj
+    if os.path.exists(out + ".key"):
+        os.remove(out + ".key")
+    os.replace(tmp, out)
+    with open(out + ".key", "w") as f:
+        f.write(key)
+
+
+def _compile(src, extra, headers, out_dir):
+    obj = os.path.join(out_dir, os.path.basename(src) + ".o")
+    key = _key(open(src, "rb").read(), headers, " ".join(_flags(src, extra)))
+    if not _fresh(obj, key):
+        _run([NVCC] + _flags(src, extra) + ["-c", src], obj, key)
+    return obj, key
 
 
 def build(verbose=False, extra=()):
-    os.makedirs(OUT_DIR, exist_ok=True)
-    srcs = sources()
+    """Compiles what is not up to date and links the library.  An object is up
+    to date by the content of its source, the headers and its flags: times say
+    nothing of flags, and the record formats that two objects share have to
+    come from one state of the headers.  Objects of other flags (``extra``) lie
+    in a folder of their own."""
+    extra = list(extra)
+    out_dir = os.path.join(OUT_DIR, "flags-" + _key(" ".join(extra))[:12]) if extra else OUT_DIR
+    os.makedirs(out_dir, exist_ok=True)
+    srcs, headers = sources(), _header_bytes()
     with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
-        objs = list(ex.map(lambda s: _compile(s, extra), srcs))
-    if (os.path.exists(LIB) and not extra
-            and os.path.getmtime(LIB) >= max(os.path.getmtime(o) for o in objs)):
-        return LIB
-    tmp = LIB + ".tmp%d" % os.getpid()
-    cmd = [NVCC] + ARCH + ["-shared", "-o", tmp] + objs
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError("link failed:\n%s\n%s" % (" ".join(cmd), r.stderr))
-    os.replace(tmp, LIB)
-    if verbose:
-        print(LIB)
+        built = list(ex.map(lambda s: _compile(s, extra, headers, out_dir), srcs))
+    key = _key(*[k for _, k in built])
+    if not _fresh(LIB, key):
+        _run([NVCC] + ARCH + ["-shared"] + [o for o, _ in built], LIB, key)
+        if verbose:
+            print(LIB)
     return LIB
 
 
