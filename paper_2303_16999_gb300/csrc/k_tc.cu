@@ -1021,6 +1021,11 @@ static_assert(kCtasPerSm * (tc_smem_bytes<false, 0>() + 1024) <= 228 * 1024 &&
                   kCtasPerSm * (tc_smem_bytes<true, 0>() + 1024) <= 228 * 1024 &&
                   kCtasPerSm * (tc_smem_bytes<true, 1>() + 1024) <= 228 * 1024,
               "two CTAs per SM");
+static_assert(tc_smem_bytes<false, 2>() <= 227 * 1024 && tc_smem_bytes<false, 3>() <= 227 * 1024 &&
+                  tc_smem_bytes<true, 2>() <= 227 * 1024 && tc_smem_bytes<true, 3>() <= 227 * 1024 &&
+                  tc_smem_bytes<false, 4>() <= 227 * 1024 && tc_smem_bytes<false, 5>() <= 227 * 1024 &&
+                  tc_smem_bytes<true, 4>() <= 227 * 1024 && tc_smem_bytes<true, 5>() <= 227 * 1024,
+              "one CTA per SM: wide and deep geometries");
 
 template <typename T, bool W8, int GEO>
 cudaError_t launch_batch(const TcBatch &B, int sm_count, cudaStream_t s) {

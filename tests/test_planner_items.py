@@ -77,3 +77,21 @@ def test_automatic_splits_stay_in_one_wave():
         cols, slots = (256, 152) if i["auto_col_tiles"] == 2 else (128, 304)
         assert i["n_items"] * -(-n // cols) <= slots, (m, k, n, b, d, i)
     assert split >= 30
+
+
+@pytest.mark.parametrize("m,k,n,b,d,kind", [
+    (4096, 16384, 24, 8, 1 / 8, "split"), (4096, 16384, 200, 8, 1 / 8, "wide split"),
+    (4096, 4096, 100, 4, 1 / 8, "split"), (4096, 4096, 1000, 4, 1 / 8, "one wave"),
+    (4096, 4096, 1000, 16, 1 / 4, "one wave"), (1024, 1024, 24, 16, 1 / 16, "rule"),
+    (4096, 4096, 2048, 16, 1 / 16, "one wave")])
+def test_shapes_by_kind(m, k, n, b, d, kind):
+    """Which shape AUTO plans take: groups split along k (over two column
+    tiles per CTA), near-equal groups that fill the SMs once, or the
+    rows-per-group rule."""
+    i = _plan(_mask(np.random.default_rng(1), m // b, k // b, "uniform", d), b, n).info()
+    split = i["n_reductions"] == i["n_groups"]
+    assert split == ("split" in kind) and (i["auto_col_tiles"] == 2) == ("wide" in kind)
+    if kind == "one wave":       # one unit per SM, or one per CTA slot
+        assert i["rows_per_group"] == 0 and i["n_items"] * -(-n // 128) in (152, 304)
+    if kind == "rule":
+        assert (i["rows_per_group"], i["n_items"]) == (1, m // 16)
