@@ -426,6 +426,27 @@ def workload_config(strong=False, world=1):
             "l2": "inputs larger than L2: 16 problems (~0.6 GB) each read once per step"}
 
 
+# The sections' tables: 17 KB of JSON.  They go to stderr, so that the result's one
+# line on stdout stays short enough for whatever keeps only the end of it.
+DETAIL = ("points", "comparators", "dynamic", "batched", "serving", "gather_small_n", "transposed",
+          "sddmm", "refit")
+
+
+def split_line(line):
+    """(the result line, its sections' tables); the line keeps the served
+    latencies at half the saturation rate, and each point's time."""
+    head = {k: v for k, v in line.items() if k not in DETAIL}
+    detail = {k: line.get(k) for k in DETAIL}
+    head["points_us"] = {"b=%d d=%s" % (p["b"], p["d"]): p["us"] for p in detail["points"] or ()}
+    srv = (detail["serving"] or {}).get("tc_fp16")
+    head["serve"] = None
+    if srv:
+        half = min(srv["rates"], key=lambda r: abs(r["rate_x_sat"] - 0.5))
+        head["serve"] = {k: half[k] for k in ("rate_x_sat", "p50_us", "p99_us")}
+        head["serve"]["saturation_rps"] = srv["saturation_rps"]
+    return head, detail
+
+
 # ------------------------------------------------------------------- main
 def main():
     ap = argparse.ArgumentParser()
@@ -645,6 +666,8 @@ def main():
                 "comparators": comparators, "dynamic": dynamic, "batched": batched,
                 "serving": serving, "gather_small_n": gsmall, "transposed": transposed,
                 "sddmm": sddmm, "refit": refit}
+        line, detail = split_line(line)
+        print(json.dumps({"detail": detail}), file=sys.stderr)
         print(json.dumps(line))
     for p in pts:
         p["plan"].close()
