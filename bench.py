@@ -908,8 +908,8 @@ def run_batched(torch, S, wl, dev, peaks, reps=5):
            "problems_on_bgather": n_bg, "problems_on_tc": len(kinds) - n_bg,
            # one BGATHER launch, one tensor-core launch per kind of CTA
            # (one or two column tiles; both stage geometries merged in each),
-           # one reduction launch per split problem
-           "gpu_launches": (1 if n_bg else 0) + tc_launches + n_red,
+           # one reduction launch for all split problems
+           "gpu_launches": (1 if n_bg else 0) + tc_launches + (1 if n_red else 0),
            "problems_on_tc_two_column_tiles": sum(wide),
            "tuner": {"buckets": len(tuned), "seconds": round(t_tune, 1), "table": tuned}}
     # the batch call as one unit: its roofline is that of all 48 problems
@@ -1016,11 +1016,12 @@ def run_gather_small_n(torch, S, wl, dev, peaks, reps=15):
     plan = S.Plan(m, k, 32, 1, w_dtype=S.F16, brow=c["brow"], bcol=c["bcol"], kernel="gather")
     plan.pack(torch.from_numpy(c["vals"].reshape(-1)).half().to(dev))
     # bytes per column index each point's kernel reads: the plan's 16-bit
-    # copy where X stays in shared memory (n = 1 and 4 at this k), else int32
-    ib16 = plan.info()["index_bytes"]
+    # copy where X stays in shared memory (n = 1 and 4 at this k, and n = 16 and
+    # 32 where the plan says so), else int32
+    info = plan.info()
 
     def idx_bytes(n):
-        return ib16 if n in (1, 4) else 4
+        return info["index_bytes"] if n in (1, 4) or info["gather_form"] else 4
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
     out = []
     for n in (1, 4, 16, 32):
