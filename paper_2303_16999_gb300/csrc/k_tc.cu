@@ -428,6 +428,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
             const int32_t e0 = it[1], e1 = it[2];
             if (e0 >= e1) continue;
             const int n0 = un.t * kNTile * G::sets;
+            const int x3 = P.x3d;   // (read once: 1 % of a dynamic call, read in every stage)
             // wide: the second column tile, unless it lies wholly past n
             const bool two = G::sets > 1 && n0 + kNTile < P.n;
             // lane l: word (l & 7) of the record, and (W producer) program word l
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                     // first warp of the tile) or one box per slab, with a 2-D
                     // map as two 64-column boxes per slab (the lower one only
                     // when the upper 64 columns lie past n)
-                    const bool joint = joint_stage<G::base>(info, P.x3d);
+                    const bool joint = joint_stage<G::base>(info, x3);
                     const int tset = (pid - 1) & 1, part = (pid - 1) >> 1;
                     const bool act = tset == 0 || two;
                     const int per = (nent + G::xprod - 1) / G::xprod;
@@ -522,13 +523,14 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                             tma_load_2d(slab + kSlabBytes / 2, &B.maps[un.p], (int)ncol + kNTile / 2,
                                         (int)xc * kTile, &sm->full[stage]);
                     }
-                } else if (joint_stage<G::base>(info, P.x3d)) {
+                } else if (joint_stage<G::base>(info, x3)) {
                     // consecutive columns: X producer 1 requests all slabs in one
                     // box, or with a 2-D map each producer those of one 64-column
                     // half (the upper one only if it holds columns of n)
                     const int x0 = n0 + (pid == 2 ? kNTile / 2 : 0);
                     const bool d3 = G::base != 0 || P.x3d;   // (as joint_stage)
-                    const uint32_t jcol = __shfl_sync(0xffffffffu, rc, 3);   // the first column
+                    // the first column (a 3-D map's box: producer 1's own first)
+                    const uint32_t jcol = G::base ? col : __shfl_sync(0xffffffffu, rc, 3);
                     if (lane == 0) {
                         if (d3 ? pid == 1 : x0 < P.n) {
                             mbar_arrive_tx(&sm->full[stage],
@@ -623,6 +625,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
             const Unit un = decode_unit(B, u);
             const int32_t *it = B.prob[un.p].items + un.item * kItemFields;
             const bool has_entries = it[2] > it[1];
+            const int x3 = B.prob[un.p].x3d;
             const bool two = G::sets > 1 && (int64_t)un.t * kNTile * G::sets + kNTile < B.prob[un.p].n;
             const int ab = local % kBufs;
             const uint32_t aphase = (local / kBufs) & 1;
@@ -649,7 +652,7 @@ __global__ void __launch_bounds__(GEO == 3 ? 416 : GEO == 2 ? 352 : kThreads, GE
                 last = (info >> 31) != 0;
                 const uint32_t myword = sm->meta[stage].prog[half][lane];   // words >= nmma unused
                 const uint32_t sbase = smem_u32(stages + stage * G::bytes);
-                const bool joint = joint_stage<G::base>(info, B.prob[un.p].x3d);
+                const bool joint = joint_stage<G::base>(info, x3);
                 const uint64_t adesc0 = joint ? a_desc_joint(sbase) : a_desc(sbase);
                 const uint32_t astep = joint ? (kSlabBytes / 2) >> 4 : kSlabBytes >> 4;
                 const uint64_t bdesc0 = b_desc(sbase + G::w16);
