@@ -199,10 +199,9 @@ static std::vector<int32_t> gx_pointers(const spmm_plan *p) {
 }
 
 // How a plan's non-zeros lie over row ranges, slices of k and rows (GxLoad).
-static GxLoad gx_load(const spmm_plan *p) {
+static GxLoad gx_load(const spmm_plan *p, const std::vector<int32_t> &ptr) {
     const HostPlan &hp = p->hp;
     const int64_t m = p->m;
-    const std::vector<int32_t> ptr = gx_pointers(p);
     GxLoad g;
     g.on = true;
     for (int64_t r = 0; r < m; ++r)
@@ -241,9 +240,10 @@ static spmm_status upload_plan(spmm_plan *p) {
     UP(d_ws_row0, ws_row0);
     if (col16_plan(p) && e == cudaSuccess) {
         // the b = 1 gather's column indices in half the bytes
-        const std::vector<uint16_t> c16(hp.col_idx.begin(), hp.col_idx.end());
-        e = upload(p, &p->d_col16, c16);
-        if (e == cudaSuccess && p->gx.on) e = upload(p, &p->d_gx_ptr, gx_pointers(p));
+        e = upload(p, &p->d_col16, p->col16);
+        if (e == cudaSuccess) e = upload(p, &p->d_gx_ptr, p->gx_ptr);
+        std::vector<uint16_t>().swap(p->col16);
+        std::vector<int32_t>().swap(p->gx_ptr);
     }
     if (p->kernel == SPMM_KERNEL_TC) {
         UP(d_grp_row0, grp_row0);
@@ -659,8 +659,12 @@ static spmm_status plan_create(int64_t m, int64_t k, int64_t n_max, int32_t b, s
                 const int64_t avg = mb ? (p->nnzb + mb - 1) / mb : 0;
                 p->C = o.max_per_item ? o.max_per_item : (int)std::max<int64_t>(64, 2 * avg);
                 build_row_plan(mb, p->C, true, p->hp);
-                // (items of a given length: the kernels that run them)
-                if (col16_plan(p) && !o.max_per_item) p->gx = gx_load(p);
+                if (col16_plan(p)) p->col16.assign(p->hp.col_idx.begin(), p->hp.col_idx.end());
+                if (col16_plan(p) && !o.max_per_item) {
+                    // (items of a given length: the kernels that run them)
+                    p->gx_ptr = gx_pointers(p);
+                    p->gx = gx_load(p, p->gx_ptr);
+                }
             } else if (kernel == SPMM_KERNEL_TC) {
                 p->groups = o.groups;
                 if (!p->groups && !o.rows_per_group && p->sm_count > 0) {

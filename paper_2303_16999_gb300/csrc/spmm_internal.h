@@ -148,7 +148,9 @@ struct spmm_plan {
     uint32_t *d_srec = nullptr, *d_sprog = nullptr;  // TC: stage records and MMA programs
     uint16_t *d_col16 = nullptr;   // static GATHER plans, k <= 65536: col_idx in 16 bits
     int32_t *d_gx_ptr = nullptr;   // with it: the first non-zero of every (row, part of k)
-    spmm::GxLoad gx;                     // what a launch of k_gather_xs.cu would find (host)
+    std::vector<uint16_t> col16;   // both on the host, until they are uploaded
+    std::vector<int32_t> gx_ptr;
+    spmm::GxLoad gx;               // what a launch of k_gather_xs.cu would find (host)
     // TC, batched with plans of the other stage geometry: this plan's stage
     // records cut for that geometry (built on first use), geometry alt_geo
     uint32_t *d_srec_alt = nullptr, *d_sprog_alt = nullptr;
