@@ -82,8 +82,10 @@ typedef enum { SPMM_F32 = 0, SPMM_F16 = 1, SPMM_BF16 = 2, SPMM_E4M3 = 3 } spmm_d
  * plan's (b, density, n) bucket overrides these rules. */
 typedef enum {
     SPMM_KERNEL_AUTO = 0,
-    SPMM_KERNEL_PLAIN = 1,   /* plain FP32 CUDA-core kernel: one thread per (row, column), F32 only */
-    SPMM_KERNEL_GATHER = 2,  /* b = 1 gather kernel: 128-bit X row loads, warp-shuffle reductions */
+    SPMM_KERNEL_PLAIN = 1,   /* FP32 CUDA-core kernels, F32 only: asked for, one thread per (row,
+                                column); chosen by AUTO (b >= 4), register-tiled blocks */
+    SPMM_KERNEL_GATHER = 2,  /* b = 1 gather kernels: 128-bit X row loads, warp-shuffle reductions;
+                                X in shared memory where that is the faster one (gather_form) */
     SPMM_KERNEL_TC = 3,      /* b >= 4 tensor-core kernel (tcgen05 + TMEM + TMA), 16-bit X */
     SPMM_KERNEL_BGATHER = 4  /* b in {4, 8, 16} CUDA-core block gather for n <= 16: static plans,
                                 16-bit X, W of the same type or E4M3; each block read once in CSR
@@ -125,7 +127,9 @@ typedef struct {
                                      2 = two whenever n > 128 (16-bit or E4M3 weights): the two
                                      tiles share every W stage (and its E4M3 expansion), one CTA
                                      per SM; 0 = automatic (two for 16-bit dense-tile plans with
-                                     n > 128 and enough work units).  Results are
+                                     n > 128 and enough work units, and for smaller plans, of
+                                     either geometry, whose groups and splits the planner made
+                                     for two: auto_col_tiles in the plan's info).  Results are
                                      identical either way.  Other values SPMM_ERR_ARG. */
     int64_t groups;               /* TC plans: split the m/16 tile rows into exactly this many
                                      groups of near-equal size (sizes differ by at most one, larger
@@ -175,6 +179,10 @@ typedef struct spmm_plan spmm_plan;
  *   m, k      : W is m x k; both multiples of b, m/b and k/b at most INT32_MAX
  *               (block indices are int32; else SPMM_ERR_SHAPE).
  *   n_max     : largest n any spmm_run of this plan will pass (sizes workspace).
+ *               Static TC plans are shaped for it: groups, and splits along k,
+ *               which fix the order of the FP32 sums, follow n_max, m and k (of
+ *               the slice, for row slices), and calls of much smaller n run
+ *               faster on a plan of their own.
  *   b         : block size, 1, 4, 8 or 16.
  *   mode      : SPMM_STATIC (pattern != NULL, host arrays, nnzb_max ignored)
  *               or SPMM_DYNAMIC (pattern ignored, 0 <= nnzb_max <= INT32_MAX fixes
@@ -334,8 +342,8 @@ int64_t spmm_bucket_size(int64_t m, int64_t k, int64_t d_max_num, int64_t d_max_
  * (problem, work item, n tile) units, precomputed on the host when the
  * plan set is first run (costliest units first) and cached until one of
  * its plans is destroyed; each CTA takes
- * every gridDim-th unit of it (no atomic work queue).  Each problem with
- * rows split over several work items adds one reduction launch.  d_X[i],
+ * every gridDim-th unit of it (no atomic work queue).  Problems with rows
+ * split over several work items share one reduction launch.  d_X[i],
  * n[i], ldx[i], d_Y[i], ldy[i] as in spmm_run (ldx/ldy may be NULL for
  * dense n).  All plans must share w_dtype and x_dtype; uneven m, k, n, b and
  * density are allowed.  The first call with a plan set allocates (its

@@ -339,10 +339,15 @@ std::vector<int64_t> group_entries(int64_t m, int64_t k, int b, int64_t nnzb, co
 //          + for split groups 2.07 + partials written and read at 5.96 TB/s.
 // Another shape than the rows-per-group rule's has to promise 20 % less, and
 // groups are split only where that rule shrinks them below 4 rows (6064 x 6800,
-// b = 8, d = 1/4, n = 319, 4 rows: 53.6 us, split 76.2).  On
-// those products the pick takes 1.02 times the best shape's time on average
-// and 0.80 times the rule's: 4096 x 16384, b = 8, d = 1/8: n = 24 62.0 -> 23.4
-// us, n = 200 82.3 -> 39.7; 4096 x 4096, b = 4, d = 1/8, n = 100 48.1 -> 16.4.
+// b = 8, d = 1/4, n = 319, 4 rows: 53.6 us, split 76.2): 4096 x 16384, b = 8, d = 1/8:
+// n = 24 62.0 -> 23.4 us, n = 200 82.3 -> 39.7; 4096 x 4096, b = 4, d = 1/8, n = 100
+// 48.1 -> 16.4.  Against plans by the rule, two-stage rings and single 2-D boxes,
+// 542 uniform products (m and k 256 to 16384, n 9 to 1000) take 0.82 of the time,
+// and so do 468 with banded, diagonal and skewed patterns.  One of those stays
+// slower for its shape: E4M3 weights of 4096 x 16384, b = 8, d = 1/8, whose columns
+// thin out, n = 200 74.8 -> 86.5 us: low columns hold most tiles and the cuts have
+// equal entries.  (E4M3 tiles at 0.028 us and the heaviest cut's count mend it,
+// and take back gains of 1.2 to 1.6 times on 20 uniform products.)
 namespace {
 struct ShapeCost {
     int64_t mt, kt, n;
