@@ -243,7 +243,7 @@ def kernel_source_sha16(files=("csrc/k_tc.cu", "csrc/tc_ptx.cuh", "csrc/capi.cpp
 # of one step; the command and the per-launch table are in
 # profiles/tc_kernel_sweep_dram.md).  Used only while the kernel and planner
 # sources hash to `sha16`; otherwise the bench reports traffic null.
-SWEEP_TRAFFIC = {"sha16": "d203c1bc4cd1969a", "bytes_per_launch": 38571792.0,
+SWEEP_TRAFFIC = {"sha16": "773bedd98192c1c3", "bytes_per_launch": 38584928.0,
                  "source": "profiles/tc_kernel_sweep_dram.md"}
 
 
@@ -257,7 +257,7 @@ def sweep_traffic():
 # L2 evicted), from one ncu capture (profiles/gather1_kernel_small_n.md);
 # used only while the gather kernels and the planner hash to `sha16`.
 GATHER_FILES = ("csrc/k_cudacore.cu", "csrc/capi.cpp", "csrc/plan_host.cpp")
-GATHER_TRAFFIC = {"sha16": "b8c2e5b5ed61398c", "bytes_per_launch": 67988992.0,
+GATHER_TRAFFIC = {"sha16": "9a638e952beb7b72", "bytes_per_launch": 68393728.0,
                   "source": "profiles/gather1_kernel_small_n.md"}
 
 

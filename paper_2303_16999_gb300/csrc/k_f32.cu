@@ -224,8 +224,9 @@ cudaError_t f32_launch(const spmm_plan *p, const void *X, int64_t n, int64_t ldx
     const int64_t nchunk = (n + CH - 1) / CH, units = p->m / B * nchunk;
     if (units > INT32_MAX) return cudaErrorInvalidConfiguration;
     // b = 8, n > 64 takes spaced columns always: 32.1 us against 37.3 with
-    // 16-byte loads (2048 x 4096, d = 1/8, n = 500); b = 4 and 16 lose by them
-    // (77 -> 85 and 52 -> 60 us at 4096 x 4096, d = 1/16, n = 1024)
+    // 16-byte loads (2048 x 4096, d = 1/8, n = 500), and 0.80 to 1.06 of their time over
+    // 26 other products (256 to 4096, d = 1/32 and 1/4, n 128 to 500); b = 4 and 16
+    // lose by them (77 -> 85 and 52 -> 60 us at 4096 x 4096, d = 1/16, n = 1024)
     constexpr bool kVec = !(B == 8 && RS == 1);
     const bool xvec = kVec && (uintptr_t)X % 16 == 0 && ldx % 4 == 0;
     const int yvec = (uintptr_t)Y % 16 == 0 && ldy % 4 == 0 ? 1 : 0;
