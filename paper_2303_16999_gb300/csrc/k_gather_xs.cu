@@ -399,7 +399,11 @@ cudaError_t gx_dispatch(const spmm_plan *p, const void *X, int64_t n, int64_t ld
 static double gx_us(const spmm_plan *p, const void *X, int64_t n, int64_t ldx, int ln, int cs) {
     const bool f32 = p->xdt == SPMM_F32;
     const int es = f32 ? 4 : 2, V = 16 / es, c = cs >> 1;   // c = log2 cs
-    const int64_t cl = cs == 1 ? gx_clusters<1>() : cs == 2 ? gx_clusters<2>() : gx_clusters<4>();
+    // (host-only plans make no CUDA calls: a GB300's 152 SMs)
+    const int64_t cl = p->host_only ? (cs == 4 ? 36 : 152 / cs)
+                       : cs == 1    ? gx_clusters<1>()
+                       : cs == 2    ? gx_clusters<2>()
+                                    : gx_clusters<4>();
     const int64_t nch = (n + ln * V - 1) / (ln * V), ranges = std::max<int64_t>(1, cl / nch);
     const int64_t rr = (p->m + ranges - 1) / ranges;
     const double waves = (double)(((p->m + rr - 1) / rr * nch + cl - 1) / cl);

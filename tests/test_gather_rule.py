@@ -42,3 +42,27 @@ def test_items_of_a_given_length_run_the_items():
     mask = _uniform(2048, 2048, 1 / 8)
     assert _form(2048, 2048, 32, mask) == 1
     assert _form(2048, 2048, 32, mask, max_per_item=64) == 0
+
+
+def test_host_only_plans_leave_the_device_alone():
+    """A process that plans on the host and asks for the plan's info holds no
+    device context afterwards (a pool may fork from it)."""
+    import subprocess
+    import sys
+    code = """
+import ctypes
+import numpy as np
+from paper_2303_16999_gb300 import spmm as S
+r, c = np.nonzero(np.random.default_rng(0).random((900, 900)) < 0.25)
+S.Plan(900, 900, 32, 1, brow=r, bcol=c, kernel="gather", host_only=True).info()
+try:
+    cu = ctypes.CDLL("libcuda.so.1")
+except OSError:
+    raise SystemExit(0)              # no driver here
+flags, active = ctypes.c_uint(), ctypes.c_int()
+st = cu.cuDevicePrimaryCtxGetState(0, ctypes.byref(flags), ctypes.byref(active))
+assert st != 0 or not active.value, (st, active.value)
+"""
+    p = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True,
+                       cwd=S.os.path.dirname(S.HERE))
+    assert p.returncode == 0, p.stderr[-2000:]
